@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "sl_internal.h"
+#include "sl_newton64.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // argument builders
@@ -115,10 +116,16 @@ template VelArgs<float> make_vel_args<float>(const sl_grid *, double, double);
 template <int DIM>
 __device__ __forceinline__ void node_coords(long long i, const int n[3], int k[3])
 {
-    k[0] = (int)(i % n[0]);
-    long long r = i / n[0];
-    k[1] = (int)(r % n[1]);
-    k[2] = DIM == 3 ? (int)(r / n[1]) : 0;
+    // a grid has fewer than 2^31 nodes: 32-bit divisions
+    const unsigned u = (unsigned)i, r = u / (unsigned)n[0];
+    k[0] = (int)(u - r * (unsigned)n[0]);
+    if (DIM == 3) {
+        k[2] = (int)(r / (unsigned)n[1]);
+        k[1] = (int)(r - (unsigned)k[2] * (unsigned)n[1]);
+    } else {
+        k[1] = (int)r;
+        k[2] = 0;
+    }
 }
 
 template <int DIM>
@@ -296,14 +303,45 @@ struct RemapDebug {
     uint8_t *status;
 };
 
+// Targets of one block: 32 x (threads / 32) nodes in 2-D, 16 x 4 x (threads / 64) in 3-D, so that
+// the stencils of a block's targets share L1 lines along every axis.  Blocks are numbered along x
+// first (grid dimensions y and z would limit the sides to 65535 blocks).
+template <int DIM>
+struct BlockShape {
+    static constexpr int X = DIM == 2 ? 32 : 16, Y3 = 4;
+    unsigned nb[3];
+    __host__ __device__ __forceinline__ BlockShape(const int n[3], unsigned threads)
+    {
+        const unsigned y = DIM == 2 ? threads / X : Y3, z = DIM == 2 ? 1 : threads / (X * Y3);
+        nb[0] = ((unsigned)n[0] + X - 1) / X;
+        nb[1] = ((unsigned)n[1] + y - 1) / y;
+        nb[2] = DIM == 2 ? 1 : ((unsigned)n[2] + z - 1) / z;
+    }
+    __device__ __forceinline__ void node(unsigned block, unsigned threads, unsigned t, int j[3]) const
+    {
+        const unsigned r = block / nb[0], bx = block - r * nb[0];
+        j[0] = (int)(bx * X + t % X);
+        if (DIM == 2) {
+            j[1] = (int)(r * (threads / X) + t / X);
+            j[2] = 0;
+        } else {
+            const unsigned bz = r / nb[1], by = r - bz * nb[1];
+            j[1] = (int)(by * Y3 + (t / X) % Y3);
+            j[2] = (int)(bz * (threads / (X * Y3)) + t / (X * Y3));
+        }
+    }
+};
+
 // NMODE: 0 = Newton in T; 1 = Newton in FP64 (FP32 data); 2 = FP32 Newton, FP64 re-solve of targets
-// whose FP32 inversion failed or whose element is close to degenerate.
+// whose FP32 inversion failed or whose element is close to degenerate.  FP64 searches (NMODE 0 of a
+// double grid, NMODE 1) run walk_seeded (sl_newton64.cuh).
 template <typename T, int DIM, int NMODE>
 __global__ void __launch_bounds__(256)
     remap_generic_kernel(GridArgs<T> g, const T *__restrict__ D, int ds, const uint8_t *__restrict__ flags,
                          FieldPtrs<T> f, RemapDebug<T> dbg, DevCounters *counters)
 {
     typedef typename std::conditional<NMODE == 1, double, T>::type TW;
+    constexpr bool SEEDED = sizeof(TW) == 8;
     LocalCounters cnt;
     cnt.clear();
     WalkParams<TW> wp;
@@ -311,10 +349,12 @@ __global__ void __launch_bounds__(256)
     wp.slack = NMODE == 1 ? TW(1e-12) : TW(g.slack);
     wp.max_iter = g.newton_max_iter;
     wp.walk_max = g.walk_max;
-    for (long long jj = blockIdx.x * (long long)blockDim.x + threadIdx.x; jj < g.N;
-         jj += (long long)gridDim.x * blockDim.x) {
-        int j[3], c[3];
-        node_coords<DIM>(jj, g.n, j);
+    int j[3], c[3];
+    const BlockShape<DIM> shape(g.n, blockDim.x);
+    shape.node(blockIdx.x, blockDim.x, threadIdx.x, j);
+    const long long jj = ((long long)j[2] * g.n[1] + j[1]) * g.n[0] + j[0];
+    // one pass (the loop only gives `continue` its meaning)
+    for (bool todo = j[0] < g.n[0] && j[1] < g.n[1] && (DIM == 2 || j[2] < g.n[2]); todo; todo = false) {
         T Dj[3] = {T(0), T(0), T(0)};
         TW xw[3] = {TW(0), TW(0), TW(0)};
 #pragma unroll
@@ -322,7 +362,11 @@ __global__ void __launch_bounds__(256)
         int hops = 0, iters = 0;
         walk_start_cell<T, DIM>(g.walk_start, j, Dj, c);
         bool degen = false;
-        int st = walk_global<T, TW, DIM>(wp, g.n, D, ds, j, c, xw, &hops, &iters, &degen);
+        int st;
+        if constexpr (SEEDED)
+            st = walk_seeded<T, DIM>(D, g.n, j, wp.max_iter, wp.walk_max, wp.tol, wp.slack, c, xw, &hops, &iters);
+        else
+            st = walk_global<T, TW, DIM>(wp, g.n, D, ds, j, c, xw, &hops, &iters, &degen);
         T xi[3] = {T(0), T(0), T(0)};
 #pragma unroll
         for (int a = 0; a < DIM; ++a) xi[a] = (T)xw[a];
@@ -400,10 +444,20 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const T x = a < DIM ? xi[a] : T(0), y = T(1) - x, x2 = x * x, y2 = y * y;
-            wc[a][0] = T(-0.5) * x * y2;
-            wc[a][1] = T(1) + x2 * (T(1.5) * x - T(2.5));
-            wc[a][2] = T(1) + y2 * (T(1.5) * y - T(2.5));
-            wc[a][3] = T(-0.5) * x2 * y;
+            if (sizeof(T) == 8) {
+                // the same cubics in 8 FP64 operations instead of 12: with p = x (1 - x),
+                // -x y^2 / 2 = -p y / 2, 1 - 5/2 x^2 + 3/2 x^3 = y + p (1 - 3/2 x) and their mirrors
+                const T p = x * y, h = T(-0.5) * p;
+                wc[a][0] = h * y;
+                wc[a][1] = y + p * (T(1) - T(1.5) * x);
+                wc[a][2] = x + p * (T(1) - T(1.5) * y);
+                wc[a][3] = h * x;
+            } else {
+                wc[a][0] = T(-0.5) * x * y2;
+                wc[a][1] = T(1) + x2 * (T(1.5) * x - T(2.5));
+                wc[a][2] = T(1) + y2 * (T(1.5) * y - T(2.5));
+                wc[a][3] = T(-0.5) * x2 * y;
+            }
             wl[a][0] = y;
             wl[a][1] = x;
         }
@@ -628,22 +682,34 @@ cudaError_t Launch<T>::remap_generic(const sl_grid *g, const void *D, const uint
     d.xi = dbg ? dbg->xi : nullptr;
     d.order = dbg ? dbg->order : nullptr;
     d.status = dbg ? dbg->status : nullptr;
-    const int blocks = grid_stride_blocks(g, g->N, 256);
-    const int nmode = sizeof(T) == 8 ? 0 : (g->desc.newton_mode == SL_NEWTON_F64 ? 1 : 2);
+    // FP64 targets keep a warp busy for microseconds: a small grid is cut into small blocks, so that
+    // its warps spread over the SMs
+    const int NT = sizeof(T) == 4 || g->N >= 256LL * 4 * g->num_sms ? 256 : 64;
+    unsigned blocks;
     if (g->dim == 2) {
-        if (nmode == 0)
-            remap_generic_kernel<T, 2, 0><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
-        else if (nmode == 1)
-            remap_generic_kernel<T, 2, 1><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
-        else
-            remap_generic_kernel<T, 2, 2><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
+        const BlockShape<2> b(ga.n, NT);
+        blocks = b.nb[0] * b.nb[1];
     } else {
-        if (nmode == 0)
-            remap_generic_kernel<T, 3, 0><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
-        else if (nmode == 1)
-            remap_generic_kernel<T, 3, 1><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
+        const BlockShape<3> b(ga.n, NT);
+        blocks = b.nb[0] * b.nb[1] * b.nb[2];
+    }
+    const bool n64 = g->desc.newton_mode == SL_NEWTON_F64;
+    const T *d0 = (const T *)D;
+    if constexpr (sizeof(T) == 8) {
+        if (g->dim == 2)
+            remap_generic_kernel<T, 2, 0><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
         else
-            remap_generic_kernel<T, 3, 2><<<blocks, 256, 0, s>>>(ga, (const T *)D, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 0><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+    } else if (g->dim == 2) {
+        if (n64)
+            remap_generic_kernel<T, 2, 1><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+        else
+            remap_generic_kernel<T, 2, 2><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+    } else {
+        if (n64)
+            remap_generic_kernel<T, 3, 1><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+        else
+            remap_generic_kernel<T, 3, 2><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
     }
     return cudaGetLastError();
 }
