@@ -242,6 +242,12 @@ __device__ __forceinline__ void walk_start_cell(int mode, const int j[3], const 
     for (int a = 0; a < DIM; ++a) {
         if (mode == SL_START_PAPER) {
             c[a] = j[a] - (Dj[a] > T(0) ? 1 : 0);
+        } else if (sizeof(T) == 8) {
+            // the same in three FP64 instructions: the conversion saturates, the clamp is an
+            // integer one, and only a NaN keeps j
+            const unsigned long long b = (unsigned long long)__double_as_longlong((double)Dj[a]) << 1;
+            const int s = __double2int_rd((double)j[a] - (double)Dj[a]);
+            c[a] = b > 0xffe0000000000000ull ? j[a] : min(max(s, j[a] - 65536), j[a] + 65536);
         } else {
             // clamped so that a garbage displacement cannot overflow the walk's integer steps
             const T s = min_t(max_t(T(j[a]) - Dj[a], T(j[a]) - T(65536)), T(j[a]) + T(65536));

@@ -29,8 +29,11 @@ namespace {
 // |det J| relative to the product of the 1-norms of J's columns (1 for a square element): above it
 // the FP32 inverse Jacobian is good to ~1e-6.
 constexpr float SEED_DET = 0.05f;
-// iterates must stay within this distance of the element for the FP32 residuals to mean much
-constexpr float SEED_REACH = 16.f;
+// Iterates must stay within this distance of the element: FP32 coordinates that far out are good to
+// 128 x 6e-8 / SEED_DET ~ 2e-4, within SEED_MARGIN.  (The failing walks at the seam of a solid-body
+// rotation meet sheared elements at coordinates of 30 to 60; with 16 here a quarter of their hops
+// took the FP64 iteration, 112 against 21 us per 64^2 step.)
+constexpr float SEED_REACH = 128.f;
 // columns of J must exceed the FP32 rounding of the vertices by this factor
 constexpr float SEED_CLEAR = 2e3f;
 // distance from a face beyond which the FP32 coordinates (good to ~1e-5) decide the step
@@ -233,7 +236,8 @@ struct Map64<3> {
 template <int DIM>
 __device__ __forceinline__ bool polish(const Map64<DIM> &m, const Seed<DIM> &s, double x[3], int *iters)
 {
-    // (x comes in as the FP32 solution, widened)
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) x[a] = widen(s.x[a]);
     for (int it = 0; it < 4; ++it) {
         float F[DIM], big = 0.f;
         m.residual(x, F);
@@ -243,7 +247,7 @@ __device__ __forceinline__ bool polish(const Map64<DIM> &m, const Seed<DIM> &s, 
             float d = 0.f;
 #pragma unroll
             for (int b = 0; b < DIM; ++b) d += s.Ji[a][b] * F[b];
-            if (!(fabsf(d) <= 0.25f)) return false;
+            if (!(fabsf(d) <= 0.2f * SEED_MARGIN)) return false;
             x[a] -= widen(d);
             big = fmaxf(big, fabsf(d));
         }
@@ -305,7 +309,10 @@ __device__ __noinline__ Solved64 solve_element64(const T *__restrict__ D, int n0
 }
 
 // Sec. 2.2 element search from element c with FP64 coordinates: the walk of the plain kernels
-// (walk_global), each element inverted as described at the top of this file.
+// (walk_global), each element inverted as described at the top of this file.  The FP32 hops run in
+// a loop of their own, so that the targets of a warp, which take different numbers of hops, do
+// their FP64 work together (polished inside the hop loop, every hop count had its own pass over
+// the FP64 code: 223 against 150 FP64 instructions per warp on a 1024^2 x 3 remap).
 template <typename T, int DIM>
 __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[3], const int j[3], int max_iter,
                                            int walk_max, double tol, double slack, int c[3], double xi[3], int *hops,
@@ -313,44 +320,59 @@ __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[
 {
     CycleCheck cyc;
     cyc.start(c[0], c[1], c[2]);
-    for (int hop = 0; hop < walk_max; ++hop) {
+    int hop = 0;
+    for (;;) {
+        // elements that the FP32 solution says are left, up to the first it cannot rule out
         T V[1 << DIM][DIM];
-        load_vertices<T, DIM>(D, n, c, V);
-        int k[3] = {c[0] - j[0], c[1] - j[1], c[2] - j[2]};
-        float P[1 << DIM][DIM], big = 1.f;
+        Seed<DIM> s;
+        int seed = SEED_NONE;
+        bool inner = false;  // inside the element by SEED_MARGIN (polishing moves x by less)
+        for (;;) {
+            if (hop >= walk_max) return ST_LOCATE;
+            load_vertices<T, DIM>(D, n, c, V);
+            float P[1 << DIM][DIM], big = 1.f;
 #pragma unroll
-        for (int v = 0; v < (1 << DIM); ++v)
+            for (int v = 0; v < (1 << DIM); ++v)
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    const float f = (float)V[v][a];
+                    big = fmaxf(big, fabsf(f));
+                    P[v][a] = (float)(c[a] + ((v >> a) & 1) - j[a]) + f;
+                }
+            seed = seed_solve(P, 1.2e-7f * big, max_iter, s);
+            ++hop;
+            *hops += 1;
+            if (seed != SEED_OK) break;
+            *iters += s.iters;
+            bool clear = true, out = false;
 #pragma unroll
             for (int a = 0; a < DIM; ++a) {
-                const float f = (float)V[v][a];
-                big = fmaxf(big, fabsf(f));
-                P[v][a] = (float)(k[a] + ((v >> a) & 1)) + f;
+                clear &= fabsf(s.x[a]) > SEED_MARGIN && fabsf(s.x[a] - 1.f) > SEED_MARGIN;
+                out |= s.x[a] < 0.f || s.x[a] > 1.f;
             }
-        Seed<DIM> s;
-        int seed = seed_solve(P, 1.2e-7f * big, max_iter, s);
-        *hops += 1;
-        int st = ST_OK, dir[3] = {0, 0, 0};
-        bool decided = false;
+            inner = clear && !out;
+            if (!clear || !out) break;  // inside, or an axis in doubt
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                c[a] += s.x[a] < 0.f ? -1 : (s.x[a] > 1.f ? 1 : 0);
+                xi[a] = widen(s.x[a]);
+            }
+            if (cyc.step(c[0], c[1], c[2])) return ST_LOCATE;
+        }
+        // this element in FP64
+        int st = ST_OK;
         if (seed == SEED_FOLD) {
 #pragma unroll
             for (int a = 0; a < DIM; ++a) xi[a] = NAN;
             return ST_FOLD;
         }
         if (seed == SEED_OK) {
-            *iters += s.iters;
-            bool clear = true;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                clear &= fabsf(s.x[a]) > SEED_MARGIN && fabsf(s.x[a] - 1.f) > SEED_MARGIN;
-                dir[a] = s.x[a] < 0.f ? -1 : (s.x[a] > 1.f ? 1 : 0);
-                xi[a] = widen(s.x[a]);
-            }
-            // clearly outside along some axis, and no axis in doubt
-            decided = clear && (dir[0] | dir[1] | dir[2]) != 0;
-            if (!decided) {
-                const Map64<DIM> m(V, k);
-                if (!polish<DIM>(m, s, xi, iters)) seed = SEED_NONE;
-            }
+            const int k[3] = {c[0] - j[0], c[1] - j[1], c[2] - j[2]};
+            const Map64<DIM> m(V, k);
+            if (!polish<DIM>(m, s, xi, iters))
+                seed = SEED_NONE;
+            else if (inner)
+                return ST_OK;
         }
         if (seed == SEED_NONE) {
             const Solved64 r = solve_element64<T, DIM>(D, n[0], n[1], n[2], c[0], c[1], c[2], j[0], j[1], j[2],
@@ -366,16 +388,14 @@ __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[
             }
             if (!finite) return st == ST_OK ? ST_NEWTON : st;
         }
-        if (!decided) {
+        int dir[3] = {0, 0, 0};
 #pragma unroll
-            for (int a = 0; a < DIM; ++a) dir[a] = xi[a] < -slack ? -1 : (xi[a] > 1.0 + slack ? 1 : 0);
-            if ((dir[0] | dir[1] | dir[2]) == 0) return st;
-        }
+        for (int a = 0; a < DIM; ++a) dir[a] = xi[a] < -slack ? -1 : (xi[a] > 1.0 + slack ? 1 : 0);
+        if ((dir[0] | dir[1] | dir[2]) == 0) return st;
 #pragma unroll
         for (int a = 0; a < DIM; ++a) c[a] += dir[a];
         if (cyc.step(c[0], c[1], c[2])) return ST_LOCATE;
     }
-    return ST_LOCATE;
 }
 
 }  // namespace
