@@ -913,6 +913,41 @@ __device__ __forceinline__ bool jump_test(T hm, T h0, T hp, T thr)
     return abs_t(dp - dm) > thr * max_t(abs_t(dp), abs_t(dm));
 }
 
+// FP64 to FP32 by bit operations, rounding towards zero; magnitudes below FP32's normal range give 0,
+// above it (infinities and NaN too) infinity.  (A conversion instruction takes an FP64 slot.)
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), a = hi & 0x7fffffffu;
+    unsigned m = __funnelshift_l((unsigned)__double2loint(x), a - 0x38000000u, 3);
+    m = a < 0x38100000u ? 0u : (a >= 0x47f00000u ? 0x7f800000u : m);
+    return __uint_as_float(m | (hi & 0x80000000u));
+}
+
+// The same test from the two differences in FP64, decided in FP32 where FP32 can: the FP64 pipe (one
+// instruction costs 64 FP32 ones) then only forms the differences, which cancel and need its digits.
+// `lo`, `hi`: the threshold less and plus a margin for the rounding of the FP32 test (4 roundings of
+// at most 1.2e-7 relative to the larger difference; the margin is 1e-6 (2 + thr)).  Between them, and for
+// differences outside the FP32 range, infinities and NaN, the test is jump_test's own.
+struct JumpBounds {
+    double thr;
+    float lo, hi;
+    __host__ __device__ explicit JumpBounds(double t)
+        : thr(t), lo((float)(t - 1e-6 * (2.0 + t))), hi((float)(t + 1e-6 * (2.0 + t)))
+    {
+    }
+};
+__device__ __forceinline__ bool jump_diffs(double dm, double dp, float fm, float fp, const JumpBounds &b)
+{
+    const float m = fmaxf(fabsf(fm), fabsf(fp)), d = fabsf(fp - fm);
+    if (m >= 1e-30f && m <= 1e30f) {
+        if (d > m * b.hi) return true;
+        if (d < m * b.lo) return false;
+    } else if (((__double_as_longlong(dm) | __double_as_longlong(dp)) << 1) == 0) {
+        return false;  // both differences are zeros: 0 > thr 0
+    }
+    return fabs(dp - dm) > b.thr * fmax(fabs(dp), fabs(dm));
+}
+
 // ------------------------------------------------------------------------------------------------
 // counters: warp + block aggregation, one global atomic per counter and block
 // ------------------------------------------------------------------------------------------------

@@ -176,6 +176,57 @@ __global__ void __launch_bounds__(256) flags_kernel(GridArgs<T> g, FieldPtrs<T> 
     }
 }
 
+// FP64 2-D flags.  A warp takes 31 columns (lane 0 is the left neighbour of lane 1, whose forward
+// difference is lane 1's backward one) and walks `rows` rows up, the forward difference of a row
+// being the backward one of the next: two FP64 subtractions per field and node where flags_kernel
+// takes four, and the test itself in FP32 (jump_diffs).  1024^2 x 3 fields: 79.8 -> 23.5 us, bound by
+// the FP64 pipe still (6.9 FP64 instructions a node).
+constexpr int FLAG_COLS = 31, FLAG_ROWS = 8;
+
+template <int NFM>
+__global__ void __launch_bounds__(128)
+    flags64_kernel(int n0, int n1, int nfields, JumpBounds b, FieldPtrs<double> f, uint8_t *__restrict__ flags,
+                   unsigned strips, unsigned nwarps, int rows)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned warp = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    if (warp >= nwarps) return;
+    const unsigned chunk = warp / strips;
+    const int x = (int)(warp - chunk * strips) * FLAG_COLS - 1 + lane;
+    const int xw = wrap_idx(x, n0), xr = wrap_near(xw + 1, n0);
+    const int y0 = (int)chunk * rows, y1 = min(y0 + rows, n1);
+    double c[NFM], dy[NFM];
+    float fy[NFM];
+#pragma unroll
+    for (int q = 0; q < NFM; ++q) {
+        if (q < nfields) {
+            c[q] = __ldg(f.in[q] + (long long)y0 * n0 + xw);
+            dy[q] = c[q] - __ldg(f.in[q] + (long long)wrap_near(y0 - 1, n1) * n0 + xw);
+            fy[q] = narrow(dy[q]);
+        }
+    }
+    for (int y = y0; y < y1; ++y) {
+        const long long row = (long long)y * n0, up = (long long)wrap_near(y + 1, n1) * n0;
+        unsigned bits = 0;
+#pragma unroll
+        for (int q = 0; q < NFM; ++q) {
+            if (q < nfields) {
+                const double u = __ldg(f.in[q] + up + xw);
+                const double dp = __ldg(f.in[q] + row + xr) - c[q], dn = u - c[q];
+                const float fp = narrow(dp), fn = narrow(dn);
+                const double dm = __shfl_up_sync(0xffffffffu, dp, 1);
+                const float fm = __shfl_up_sync(0xffffffffu, fp, 1);
+                if (lane > 0 && (jump_diffs(dm, dp, fm, fp, b) || jump_diffs(dy[q], dn, fy[q], fn, b)))
+                    bits |= 1u << q;
+                c[q] = u;
+                dy[q] = dn;
+                fy[q] = fn;
+            }
+        }
+        if (lane > 0 && x < n0) flags[row + x] = (uint8_t)bits;
+    }
+}
+
 // ------------------------------------------------------------------------------------------------
 // eq. (vel): RK4 displacement of every Lagrangian node (cell units), stride ds values per node
 // ------------------------------------------------------------------------------------------------
@@ -670,6 +721,25 @@ cudaError_t Launch<T>::flags(const sl_grid *g, const void *const *in, uint8_t *f
     const GridArgs<T> ga = make_grid_args<T>(g);
     const FieldPtrs<T> f = field_ptrs<T>(g, in, nullptr);
     const int blocks = grid_stride_blocks(g, g->N, 256);
+    if constexpr (sizeof(T) == 8) {
+        if (g->dim == 2 && g->desc.limiter_threshold >= 0.0) {
+            const unsigned strips = (unsigned)((g->n[0] + FLAG_COLS - 1) / FLAG_COLS);
+            // fewer rows a warp where the grid has too few warps to fill the SMs: a row takes ~1 us of
+            // dependent FP64 latency, which only other warps can hide
+            const int rows = strips * (g->n[1] / FLAG_ROWS) >= 8u * g->num_sms ? FLAG_ROWS : 1;
+            const unsigned nwarps = strips * (unsigned)((g->n[1] + rows - 1) / rows);
+            const JumpBounds b(g->desc.limiter_threshold);
+            const int n0 = (int)g->n[0], n1 = (int)g->n[1], nf = g->nfields;
+            const unsigned nb = (nwarps + 3) / 4;
+            if (nf == 1)
+                flags64_kernel<1><<<nb, 128, 0, s>>>(n0, n1, nf, b, f, flags, strips, nwarps, rows);
+            else if (nf <= 4)
+                flags64_kernel<4><<<nb, 128, 0, s>>>(n0, n1, nf, b, f, flags, strips, nwarps, rows);
+            else
+                flags64_kernel<8><<<nb, 128, 0, s>>>(n0, n1, nf, b, f, flags, strips, nwarps, rows);
+            return cudaGetLastError();
+        }
+    }
     if (g->dim == 2)
         flags_kernel<T, 2><<<blocks, 256, 0, s>>>(ga, f, flags);
     else
