@@ -162,6 +162,27 @@ __device__ __forceinline__ float recip_t(float x)
 }
 __device__ __forceinline__ double recip_t(double x) { return 1.0 / x; }
 
+// FP64 to FP32 by bit operations, rounding towards zero; magnitudes below FP32's normal range give 0,
+// above it (infinities and NaN too) infinity.  (A conversion instruction takes an FP64 slot.)
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), a = hi & 0x7fffffffu;
+    unsigned m = __funnelshift_l((unsigned)__double2loint(x), a - 0x38000000u, 3);
+    m = a < 0x38100000u ? 0u : (a >= 0x47f00000u ? 0x7f800000u : m);
+    return __uint_as_float(m | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float narrow(float x) { return x; }
+
+// FP32 to FP64, exact, by bit operations; |f| below the normal range counts as zero
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    if (m < 0x00800000u) return 0.0;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+// |k| < 2^24
+__device__ __forceinline__ double small_int(int k) { return widen((float)k); }
+
 __device__ __forceinline__ void sincospi_t(double x, double *s, double *c) { sincospi(x, s, c); }
 // FP32 sin(pi x), cos(pi x): x = q/2 + r with q = rint(2x) and |r| <= 1/4 (both exact), the Taylor
 // series of sin(pi r) through r^9 and of cos(pi r) through r^10 (truncation below 2e-9 for
@@ -911,16 +932,6 @@ __device__ __forceinline__ bool jump_test(T hm, T h0, T hp, T thr)
 {
     const T dp = hp - h0, dm = h0 - hm;
     return abs_t(dp - dm) > thr * max_t(abs_t(dp), abs_t(dm));
-}
-
-// FP64 to FP32 by bit operations, rounding towards zero; magnitudes below FP32's normal range give 0,
-// above it (infinities and NaN too) infinity.  (A conversion instruction takes an FP64 slot.)
-__device__ __forceinline__ float narrow(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x), a = hi & 0x7fffffffu;
-    unsigned m = __funnelshift_l((unsigned)__double2loint(x), a - 0x38000000u, 3);
-    m = a < 0x38100000u ? 0u : (a >= 0x47f00000u ? 0x7f800000u : m);
-    return __uint_as_float(m | (hi & 0x80000000u));
 }
 
 // The same test from the two differences in FP64, decided in FP32 where FP32 can: the FP64 pipe (one

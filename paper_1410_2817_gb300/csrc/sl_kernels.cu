@@ -372,7 +372,7 @@ __device__ __forceinline__ void walk_start_cell(int mode, const int j[3], const 
             // the same in three FP64 instructions: the conversion saturates, the clamp is an
             // integer one, and only a NaN keeps j
             const unsigned long long b = (unsigned long long)__double_as_longlong((double)Dj[a]) << 1;
-            const int s = __double2int_rd((double)j[a] - (double)Dj[a]);
+            const int s = __double2int_rd(small_int(j[a]) - (double)Dj[a]);
             c[a] = b > 0xffe0000000000000ull ? j[a] : min(max(s, j[a] - 65536), j[a] + 65536);
         } else {
             // clamped so that a garbage displacement cannot overflow the walk's integer steps
@@ -467,7 +467,9 @@ struct BlockShape {
 // NMODE: 0 = Newton in T; 1 = Newton in FP64 (FP32 data); 2 = FP32 Newton, FP64 re-solve of targets
 // whose FP32 inversion failed or whose element is close to degenerate.  FP64 searches (NMODE 0 of a
 // double grid, NMODE 1) run walk_seeded (sl_newton64.cuh).
-template <typename T, int DIM, int NMODE>
+// QUINTIC: the grid may take order 2 (without it the kernel carries none of its code: the compiler
+// hoists the quintic weights out of the fields' loop, 34 FP64 instructions a target; 331 -> 264 us).
+template <typename T, int DIM, int NMODE, bool QUINTIC>
 __global__ void __launch_bounds__(256)
     remap_generic_kernel(GridArgs<T> g, const T *__restrict__ D, int ds, const uint8_t *__restrict__ flags,
                          FieldPtrs<T> f, RemapDebug<T> dbg, DevCounters *counters)
@@ -481,6 +483,10 @@ __global__ void __launch_bounds__(256)
     wp.slack = NMODE == 1 ? TW(1e-12) : TW(g.slack);
     wp.max_iter = g.newton_max_iter;
     wp.walk_max = g.walk_max;
+    // The cubic weights of an FP64 target wait in shared memory for the fields' sums: kept in registers,
+    // the compiler saves those by forming the weights again for every field (18 FP64 instructions of 38;
+    // 1024^2 x 3 fields: 386 -> 331 us).
+    __shared__ volatile double sw[sizeof(T) == 8 ? DIM * 4 : 1][sizeof(T) == 8 ? 256 : 1];
     int j[3], c[3];
     const BlockShape<DIM> shape(g.n, blockDim.x);
     shape.node(blockIdx.x, blockDim.x, threadIdx.x, j);
@@ -549,14 +555,15 @@ __global__ void __launch_bounds__(256)
         constexpr int KZ = DIM == 3 ? 4 : 1;
         // Sec. 2.3: OR of the flag bytes over the stencils of order 2 ([c-2, c+3]) and 1 ([c-1, c+2])
         unsigned box2 = 0, box1 = 0;
-        if (g.max_order == 1) {
+        const int max_order = QUINTIC ? g.max_order : min(g.max_order, 1);
+        if (max_order == 1) {
 #pragma unroll
             for (int kz = 0; kz < KZ; ++kz)
 #pragma unroll
                 for (int ky = 0; ky < 4; ++ky)
 #pragma unroll
                     for (int kx = 0; kx < 4; ++kx) box1 |= __ldg(flags + oz[kz] + oy[ky] + ox[kx]);
-        } else if (g.max_order >= 2) {
+        } else if (QUINTIC && max_order >= 2) {
             const int r = 2, w = 6;
             const int cnt_box = DIM == 3 ? w * w * w : w * w;
             for (int q = 0; q < cnt_box; ++q) {
@@ -572,10 +579,10 @@ __global__ void __launch_bounds__(256)
         }
         // eq. (multiZ) weights of orders 1 (Z~1 at taps c-1 .. c+2, Appendix) and 0 (hat at c, c+1),
         // once per target
-        T wc[3][4], wl[3][2];
+        T wc[DIM][4], wl[DIM][2];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const T x = a < DIM ? xi[a] : T(0), y = T(1) - x, x2 = x * x, y2 = y * y;
+        for (int a = 0; a < DIM; ++a) {
+            const T x = xi[a], y = T(1) - x, x2 = x * x, y2 = y * y;
             if (sizeof(T) == 8) {
                 // the same cubics in 8 FP64 operations instead of 12: with p = x (1 - x),
                 // -x y^2 / 2 = -p y / 2, 1 - 5/2 x^2 + 3/2 x^3 = y + p (1 - 3/2 x) and their mirrors
@@ -592,10 +599,15 @@ __global__ void __launch_bounds__(256)
             }
             wl[a][0] = y;
             wl[a][1] = x;
+            if (sizeof(T) == 8) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) sw[a * 4 + k][threadIdx.x] = wc[a][k];
+            }
         }
+        auto weight = [&](int a, int k) -> T { return sizeof(T) == 8 ? (T)sw[a * 4 + k][threadIdx.x] : wc[a][k]; };
         for (int q = 0; q < g.nfields; ++q) {
-            int m = g.max_order;
-            if (m == 2 && ((box2 >> q) & 1u)) m = 1;
+            int m = max_order;
+            if (QUINTIC && m == 2 && ((box2 >> q) & 1u)) m = 1;
             if (m >= 1 && ((box1 >> q) & 1u)) m = 0;
             cnt.oh0 += m == 0;
             cnt.oh1 += m == 1;
@@ -604,31 +616,39 @@ __global__ void __launch_bounds__(256)
             const T *h = f.in[q];
             T sum = T(0);
             if (m == 1) {
-#pragma unroll
-                for (int kz = 0; kz < KZ; ++kz) {
-                    T sy = T(0);
-#pragma unroll
-                    for (int ky = 0; ky < 4; ++ky) {
-                        const T *row = h + oz[kz] + oy[ky];
-                        T sx = T(0);
-#pragma unroll
-                        for (int kx = 0; kx < 4; ++kx) sx += wc[0][kx] * __ldg(row + ox[kx]);
-                        sy += wc[1][ky] * sx;
-                    }
-                    sum += (DIM == 3 ? wc[2][kz] : T(1)) * sy;
+                // rows of four taps, rows into a plane, planes into the sum
+                auto row = [&](int kz, int ky) {
+                    const T *r = h + oz[kz] + oy[ky];
+                    T v = mul_rn_t(weight(0, 0), __ldg(r + ox[0]));
+                    v = fma_rn_t(weight(0, 1), __ldg(r + ox[1]), v);
+                    v = fma_rn_t(weight(0, 2), __ldg(r + ox[2]), v);
+                    return fma_rn_t(weight(0, 3), __ldg(r + ox[3]), v);
+                };
+                auto plane = [&](int kz) {
+                    T v = mul_rn_t(weight(1, 0), row(kz, 0));
+                    v = fma_rn_t(weight(1, 1), row(kz, 1), v);
+                    v = fma_rn_t(weight(1, 2), row(kz, 2), v);
+                    return fma_rn_t(weight(1, 3), row(kz, 3), v);
+                };
+                if constexpr (DIM == 2) {
+                    sum = plane(0);
+                } else {
+                    sum = mul_rn_t(weight(2, 0), plane(0));
+                    sum = fma_rn_t(weight(2, 1), plane(1), sum);
+                    sum = fma_rn_t(weight(2, 2), plane(2), sum);
+                    sum = fma_rn_t(weight(2, 3), plane(3), sum);
                 }
             } else if (m == 0) {
-#pragma unroll
-                for (int kz = 0; kz < (DIM == 3 ? 2 : 1); ++kz) {
-                    T sy = T(0);
-#pragma unroll
-                    for (int ky = 0; ky < 2; ++ky) {
-                        const T *row = h + oz[kz + 1] + oy[ky + 1];
-                        sy += wl[1][ky] * (wl[0][0] * __ldg(row + ox[1]) + wl[0][1] * __ldg(row + ox[2]));
-                    }
-                    sum += (DIM == 3 ? wl[2][kz] : T(1)) * sy;
-                }
-            } else {
+                auto row = [&](int kz, int ky) {
+                    const T *r = h + oz[kz] + oy[ky];
+                    return fma_rn_t(wl[0][1], __ldg(r + ox[2]), mul_rn_t(wl[0][0], __ldg(r + ox[1])));
+                };
+                auto plane = [&](int kz) { return fma_rn_t(wl[1][1], row(kz, 2), mul_rn_t(wl[1][0], row(kz, 1))); };
+                if constexpr (DIM == 2)
+                    sum = plane(0);
+                else
+                    sum = fma_rn_t(wl[2][1], plane(2), mul_rn_t(wl[2][0], plane(1)));
+            } else if (QUINTIC) {
                 T w[3][6];
 #pragma unroll
                 for (int a = 0; a < DIM; ++a) zs_weights<T>(m, xi[a], w[a]);
@@ -863,20 +883,25 @@ cudaError_t Launch<T>::remap_generic(const sl_grid *g, const void *D, const uint
     const bool n64 = g->desc.newton_mode == SL_NEWTON_F64;
     const T *d0 = (const T *)D;
     if constexpr (sizeof(T) == 8) {
-        if (g->dim == 2)
-            remap_generic_kernel<T, 2, 0><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+        const bool z2 = g->desc.max_order > 1;
+        if (g->dim == 2 && z2)
+            remap_generic_kernel<T, 2, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+        else if (g->dim == 2)
+            remap_generic_kernel<T, 2, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+        else if (z2)
+            remap_generic_kernel<T, 3, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
         else
-            remap_generic_kernel<T, 3, 0><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
     } else if (g->dim == 2) {
         if (n64)
-            remap_generic_kernel<T, 2, 1><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
         else
-            remap_generic_kernel<T, 2, 2><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
     } else {
         if (n64)
-            remap_generic_kernel<T, 3, 1><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
         else
-            remap_generic_kernel<T, 3, 2><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
     }
     return cudaGetLastError();
 }

@@ -13,6 +13,10 @@
 //     inverse Jacobian Ji in FP32, which gains ~6 digits per pass (two passes as a rule, 12 / 42
 //     FP64 instructions in 2-D / 3-D), down to the rounding error of F, as the FP64 iteration does.
 //
+// Conversions between FP32, FP64 and integers take an FP64 slot too and are done by bit operations.
+// A 1024^2 x 3 remap issues 113 FP64 instructions per warp where the all-FP64 search needed 263 a target:
+// 480 -> 223 us; 64^3 x 2 fields 640 -> 145 us.
+//
 // Every decision of the FP64 search (fold, no convergence, inside, next element) is taken from the
 // FP32 solution only under a certificate (seed_solve): Jacobian determinants at every iterate well
 // away from zero, iterates that stay near the element, convergence with iterations to spare.  Then
@@ -35,7 +39,7 @@ constexpr float SEED_DET = 0.05f;
 // took the FP64 iteration, 112 against 21 us per 64^2 step.)
 constexpr float SEED_REACH = 128.f;
 // columns of J must exceed the FP32 rounding of the vertices by this factor
-constexpr float SEED_CLEAR = 2e3f;
+constexpr float SEED_CLEAR = 1e3f;
 // distance from a face beyond which the FP32 coordinates (good to ~1e-5) decide the step
 constexpr float SEED_MARGIN = 1e-3f;
 // iterations the FP64 solve needs beyond the FP32 one: 3e-4 -> 1e-7 -> 1e-14 -> below its 1e-14 stop
@@ -49,15 +53,6 @@ struct Seed {
     float Ji[DIM][DIM];  // inverse Jacobian there
     int iters;
 };
-
-// exact widening by bit operations (a conversion instruction would take an FP64 slot); |f| below
-// the normal range counts as zero
-__device__ __forceinline__ double widen(float f)
-{
-    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
-    if (m < 0x00800000u) return 0.0;
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-}
 
 // FP32 Newton inversion of the bilinear element with vertices P (relative to the target, rounded to
 // within `noise`), the iteration of newton_solve2 under the certificate described above.
@@ -183,7 +178,7 @@ struct Map64<2> {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const double v0 = (double)V[0][q], v1 = (double)V[1][q], d20 = (double)V[2][q] - v0;
-            p[q] = (double)k[q] + v0;
+            p[q] = small_int(k[q]) + v0;
             a[q] = v1 - v0;
             e[q] = ((double)V[3][q] - v1) - d20;
             b[q] = d20;
@@ -194,7 +189,7 @@ struct Map64<2> {
     __device__ __forceinline__ void residual(const double x[3], float F[2]) const
     {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) F[q] = (float)fma(x[1], fma(x[0], e[q], b[q]), fma(x[0], a[q], p[q]));
+        for (int q = 0; q < 2; ++q) F[q] = narrow(fma(x[1], fma(x[0], e[q], b[q]), fma(x[0], a[q], p[q])));
     }
 };
 template <>
@@ -208,7 +203,7 @@ struct Map64<3> {
             const double v0 = (double)V[0][q], v2 = (double)V[2][q], v4 = (double)V[4][q], v6 = (double)V[6][q];
             const double d10 = (double)V[1][q] - v0, d32 = (double)V[3][q] - v2, d54 = (double)V[5][q] - v4,
                          d76 = (double)V[7][q] - v6;
-            p[q] = (double)k[q] + v0;
+            p[q] = small_int(k[q]) + v0;
             a[q] = d10;
             b[q] = v2 - v0;
             c[q] = v4 - v0;
@@ -226,7 +221,7 @@ struct Map64<3> {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const double u = fma(x[1], fma(x[2], g[q], e01[q]), fma(x[2], e02[q], a[q]));
-            F[q] = (float)fma(x[0], u, fma(x[1], fma(x[2], e12[q], b[q]), fma(x[2], c[q], p[q])));
+            F[q] = narrow(fma(x[0], u, fma(x[1], fma(x[2], e12[q], b[q]), fma(x[2], c[q], p[q]))));
         }
     }
 };
@@ -335,11 +330,11 @@ __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[
             for (int v = 0; v < (1 << DIM); ++v)
 #pragma unroll
                 for (int a = 0; a < DIM; ++a) {
-                    const float f = (float)V[v][a];
+                    const float f = narrow(V[v][a]);
                     big = fmaxf(big, fabsf(f));
                     P[v][a] = (float)(c[a] + ((v >> a) & 1) - j[a]) + f;
                 }
-            seed = seed_solve(P, 1.2e-7f * big, max_iter, s);
+            seed = seed_solve(P, 2.4e-7f * big, max_iter, s);
             ++hop;
             *hops += 1;
             if (seed != SEED_OK) break;
