@@ -123,7 +123,10 @@ typedef struct {
     int fail_policy;                /* SL_FAIL_KEEP or SL_FAIL_ERROR                                  */
     int walk_start;                 /* SL_START_BACKWARD (from j - D_j) or SL_START_PAPER (Sec. 2.2) */
     int kernel;                     /* SL_KERNEL_AUTO, SL_KERNEL_GENERIC or SL_KERNEL_TILED           */
-    int tile_config;                /* 2-D FP32 tiles: 0 default (7 where it applies, else 1);
+    int tile_config;                /* 2-D FP32 kernel: 0 default (up to 4 fields and max_order <= 1:
+                                       the two-phase kernel, which flags every node once and
+                                       gathers through L1, or 1, whichever is the faster one for
+                                       the size; else 1);
                                        6: 64x32 and 7: 32x32 tiles of the persistent kernel whose
                                        windows are copied by TMA boxes (one CTA per SM with 6, two
                                        with 7; up to 3 fields, max_order <= 1, an analytic velocity,

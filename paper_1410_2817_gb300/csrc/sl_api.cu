@@ -114,8 +114,16 @@ static const char *check_desc(const sl_grid_desc *d)
 }
 
 struct Layout {
-    size_t counters, stripes, trig, partials, moment_out, flags, flags2, D0, D1, rk, total;
+    size_t counters, stripes, sync, trig, partials, moment_out, flags, flags2, D0, D1, rk, rec, total;
 };
+
+// Does the grid run the two-phase 2-D FP32 step (whose records the workspace holds)?
+static bool has_records(const sl_grid_desc *d)
+{
+    return d->dim == 2 && d->dtype == SL_F32 && d->max_order <= 1 && d->nfields <= 4 && d->newton_mode == SL_NEWTON_MIXED &&
+           d->walk_start == SL_START_BACKWARD && d->kernel != SL_KERNEL_GENERIC && d->tile_config == 0 &&
+           (d->n[0] + 3) * (d->n[1] + 3) < (1LL << 31);  // 32-bit record indices
+}
 
 static Layout layout_of(const sl_grid_desc *d)
 {
@@ -129,6 +137,8 @@ static Layout layout_of(const sl_grid_desc *d)
     off += align256(sizeof(DevCounters));
     L.stripes = off;
     off += align256(sizeof(DevCounters) * SL_COUNTER_STRIPES);
+    L.sync = off;
+    off += 256;
     L.trig = off;
     if (d->velocity_kind == SL_VEL_SWIRL2D || d->velocity_kind == SL_VEL_DEFORM3D) {
         long long nt = 0;
@@ -151,6 +161,8 @@ static Layout layout_of(const sl_grid_desc *d)
     // viscous stress (13 planes)
     L.rk = off;
     if (d->velocity_kind == SL_VEL_NLSW) off += align256((size_t)N * 13 * ts);
+    L.rec = off;
+    if (has_records(d)) off += gather2d_record_bytes(d->n[0], d->n[1], d->nfields);
     L.total = off;
     return L;
 }
@@ -209,6 +221,8 @@ extern "C" sl_status sl_create_grid(const sl_grid_desc *desc, void *dev_workspac
     g->moment_out = (double *)(g->ws + L.moment_out);
     g->flags = (uint8_t *)(g->ws + L.flags);
     g->flags2 = (uint8_t *)(g->ws + L.flags2);
+    g->rec = has_records(desc) ? (void *)(g->ws + L.rec) : nullptr;
+    g->sync = (unsigned *)(g->ws + L.sync);
     g->D[0] = g->ws + L.D0;
     g->D[1] = g->ws + L.D1;
     g->dcur = 0;

@@ -27,6 +27,8 @@ struct sl_grid {
     double *moment_out;          // 8 doubles
     uint8_t *flags;              // N
     uint8_t *flags2;             // N (second byte buffer: separable OR of flags over stencils)
+    void *rec;                   // records of the two-phase 2-D FP32 step (null where it does not run)
+    unsigned *sync;              // its phase counters (zero between launches)
     void *D[2];                  // two displacement buffers (ping-pong for the pipelined step)
     int dcur;                    // index of the current displacement
     int device, num_sms;
@@ -106,6 +108,10 @@ size_t tiled2d_smem_bytes_cfgd(int nfields);
 // shallow water (sl_nlsw.cu): the viscosity nu of a grid and the launches of one step's stages
 double nlsw_viscosity(const sl_grid *g);
 int nlsw_kernels_per_step(const sl_grid *g);
+// 2-D FP32 step in two phases over flagged records (sl_gather2d.cu): tile configuration 0
+size_t gather2d_record_bytes(long long n0, long long n1, int nfields);
+cudaError_t launch_gather2d(const sl_grid *g, const void *D, void *D_next, double t_next, double dt, bool fused,
+                            const void *const *in, void *const *out, cudaStream_t s);
 // 2-D FP32 persistent remap with TMA-staged windows (sl_remap2d.cu): configuration 6 (64x32 tiles,
 // one CTA per SM) or 7 (32x32 tiles, two CTAs per SM)
 bool remap2d_tma_supported(const sl_grid *g, const void *const *in, void *const *out);
