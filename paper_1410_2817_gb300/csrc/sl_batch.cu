@@ -30,7 +30,7 @@ struct BatchGrid {
     double dt, period;             // period > 0: time-dependent velocity cos(pi t / period)
     int dcur;                      // displacement buffer holding D at the call's first step
     int steady;                    // steady velocity: D of the first step serves every step
-    int tiles_x, tile_base;
+    int tiles_x, tile_base, ntiles;
 };
 
 // cos(pi t / period) at the stage times of every trajectory sub-step of a step starting at t, by
@@ -137,32 +137,67 @@ __global__ void __launch_bounds__(CfgZ::NT, CfgZ::MINB)
     }
 }
 
+// The trajectory and the finishing kernel claim runs of up to RUN_TILES consecutive tiles of one grid: claimed
+// tile by tile they are bound by the counter (~6 ns a claim, 25,000 tiles in 512 grids of 24.4 M nodes).
+// Longer runs leave CTAs idle at the end.  The finishing copy: 138 -> 100 us.
+constexpr int RUN_TILES = 2;
+// CTAs per SM of the trajectory kernel's register budget (2 / 3 / 4: 773 / 702 / 724 us)
+constexpr int ADVB = 3;
+
+struct Run {
+    int grid, tile, count;
+};
+
 // RK4 displacements of every grid's nodes at the grid's time (before the first step of a call)
 template <class Cfg>
-__global__ void __launch_bounds__(Cfg::NT)
-    batch_advect_kernel(const BatchGrid *__restrict__ table, const int *__restrict__ item_grid, int nitems,
-                        unsigned *counter, const double *__restrict__ tgrid)
+__global__ void __launch_bounds__(Cfg::NT, ADVB)
+    batch_advect_kernel(const BatchGrid *__restrict__ table, const Run *__restrict__ runs, int nruns, unsigned *counter,
+                        const double *__restrict__ tgrid)
 {
     __shared__ int s_item;
     __shared__ __align__(16) BatchGrid sg;
     __shared__ VelArgs<float> sv;
-    for (int item = next_item(counter, &s_item); item < nitems; item = next_item(counter, &s_item)) {
-        const int gid = __ldg(item_grid + item);
+    __shared__ FourierPairs sf;
+    __shared__ float4 base[SL_PAIR_MODES][Cfg::NT];
+    for (int run = next_item(counter, &s_item); run < nruns; run = next_item(counter, &s_item)) {
+        const int gid = __ldg(&runs[run].grid), tile0 = __ldg(&runs[run].tile), count = __ldg(&runs[run].count);
         load_entry(table, gid, &sg);
         if (threadIdx.x == 0) {
             sv = sg.vel;
             stage_factors(sg, tgrid[gid], sv.ct);
         }
         __syncthreads();
-        const int t = item - sg.tile_base;
-        const int ty = t / sg.tiles_x, tx = t - ty * sg.tiles_x;
+        const bool pairs = fourier2d_pairs(sv);
+        if (pairs) {
+            sf.load(sv, threadIdx.x);
+            __syncthreads();
+        }
         float2 *D = reinterpret_cast<float2 *>(sg.D[sg.dcur]);
-        for (int q = threadIdx.x; q < Cfg::TX * Cfg::TY; q += Cfg::NT) {
-            const int jx = tx * Cfg::TX + q % Cfg::TX, jy = ty * Cfg::TY + q / Cfg::TX;
-            if (jx >= sg.base.n0 || jy >= sg.base.n1) continue;
-            float X[3] = {node_position(sv.lo[0], jx, sv.dx[0]), node_position(sv.lo[1], jy, sv.dx[1]), 0.f}, d[3];
-            trajectory_cells<float, 2>(sv, X, d);
-            D[(long long)jy * sg.base.n0 + jx] = make_float2(d[0], d[1]);
+        const int n0 = sg.base.n0, n1 = sg.base.n1;
+        for (int t = tile0; t < tile0 + count; ++t) {
+            const int ty = t / sg.tiles_x, tx = t - ty * sg.tiles_x;
+            if (pairs) {
+                // two nodes a thread, half a tile apart (the code of a grid alone)
+                constexpr int H = Cfg::TX * Cfg::TY / 2;
+                for (int q = threadIdx.x; q < H; q += Cfg::NT) {
+                    const int jx = tx * Cfg::TX + q % Cfg::TX, ja = ty * Cfg::TY + q / Cfg::TX, jb = ja + Cfg::TY / 2;
+                    if (jx >= n0 || ja >= n1) continue;
+                    const float x = node_position(sv.lo[0], jx, sv.dx[0]);
+                    const float2 Y = make_float2(node_position(sv.lo[1], ja, sv.dx[1]), node_position(sv.lo[1], jb, sv.dx[1]));
+                    float2 Dx, Dy;
+                    rk4_fourier2d_pair(sf, &base[0][threadIdx.x], Cfg::NT, make_float2(x, x), Y, Dx, Dy);
+                    D[(unsigned)ja * (unsigned)n0 + (unsigned)jx] = make_float2(Dx.x, Dy.x);
+                    if (jb < n1) D[(unsigned)jb * (unsigned)n0 + (unsigned)jx] = make_float2(Dx.y, Dy.y);
+                }
+                continue;
+            }
+            for (int q = threadIdx.x; q < Cfg::TX * Cfg::TY; q += Cfg::NT) {
+                const int jx = tx * Cfg::TX + q % Cfg::TX, jy = ty * Cfg::TY + q / Cfg::TX;
+                if (jx >= n0 || jy >= n1) continue;
+                float X[3] = {node_position(sv.lo[0], jx, sv.dx[0]), node_position(sv.lo[1], jy, sv.dx[1]), 0.f}, d[3];
+                trajectory_cells<float, 2>(sv, X, d);
+                D[(unsigned)jy * (unsigned)n0 + (unsigned)jx] = make_float2(d[0], d[1]);
+            }
         }
     }
 }
@@ -170,33 +205,41 @@ __global__ void __launch_bounds__(Cfg::NT)
 // after a call: fields back into the caller's planes (odd step counts) and the grids' times
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::NT)
-    batch_finish_kernel(const BatchGrid *__restrict__ table, const int *__restrict__ item_grid, int nitems,
-                        unsigned *counter, double *tgrid, int ngrids, int nsteps)
+    batch_finish_kernel(const BatchGrid *__restrict__ table, const Run *__restrict__ runs, int nruns, unsigned *counter,
+                        double *tgrid, int ngrids, int nsteps)
 {
     __shared__ int s_item;
-    __shared__ __align__(16) BatchGrid sg;
     if (blockIdx.x == 0)
         for (int g = threadIdx.x; g < ngrids; g += blockDim.x) tgrid[g] += (double)nsteps * table[g].dt;
     if ((nsteps & 1) == 0) return;
-    for (int item = next_item(counter, &s_item); item < nitems; item = next_item(counter, &s_item)) {
-        const int gid = __ldg(item_grid + item);
-        load_entry(table, gid, &sg);
-        const int t = item - sg.tile_base;
-        const int ty = t / sg.tiles_x, tx = t - ty * sg.tiles_x;
-        for (int q = threadIdx.x; q < Cfg::TX * Cfg::TY; q += Cfg::NT) {
-            const int jx = tx * Cfg::TX + q % Cfg::TX, jy = ty * Cfg::TY + q / Cfg::TX;
-            if (jx >= sg.base.n0 || jy >= sg.base.n1) continue;
-            const long long jj = (long long)jy * sg.base.n0 + jx;
-            for (int f = 0; f < sg.base.nfields; ++f) const_cast<float *>(sg.fields[f])[jj] = sg.scratch[f][jj];
+    for (int run = next_item(counter, &s_item); run < nruns; run = next_item(counter, &s_item)) {
+        const BatchGrid &g = table[__ldg(&runs[run].grid)];
+        const int tile0 = __ldg(&runs[run].tile), count = __ldg(&runs[run].count);
+        // the run's share of every plane: a contiguous piece, 16 bytes at a time where the planes allow
+        const unsigned N = (unsigned)g.base.n0 * (unsigned)g.base.n1, nt = (unsigned)g.ntiles;
+        const unsigned per = ((N + nt - 1) / nt + 3u) & ~3u;
+        const unsigned lo = min(N, per * (unsigned)tile0), hi = min(N, per * (unsigned)(tile0 + count));
+        const int nf = g.base.nfields;
+        for (int f = 0; f < nf; ++f) {
+            float *dst = const_cast<float *>(g.fields[f]);
+            const float *src = g.scratch[f];
+            unsigned i = lo + threadIdx.x;
+            if ((((uintptr_t)dst | (uintptr_t)src) & 15u) == 0) {
+                const unsigned v1 = hi / 4;
+                for (unsigned v = lo / 4 + threadIdx.x; v < v1; v += Cfg::NT)
+                    reinterpret_cast<float4 *>(dst)[v] = __ldcs(reinterpret_cast<const float4 *>(src) + v);
+                i = max(lo, v1 * 4) + threadIdx.x;
+            }
+            for (; i < hi; i += Cfg::NT) dst[i] = src[i];
         }
     }
 }
 
 struct BatchLayout {
-    size_t table, items, counters, tgrid, total;
+    size_t table, items, counters, tgrid, runs, total;
 };
 
-BatchLayout batch_layout(int count, int nitems)
+BatchLayout batch_layout(int count, int nitems, int nruns)
 {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     BatchLayout L;
@@ -209,6 +252,8 @@ BatchLayout batch_layout(int count, int nitems)
     off += al(sizeof(unsigned) * (SL_BATCH_MAX_STEPS + 2));
     L.tgrid = off;
     off += al(sizeof(double) * (size_t)count);
+    L.runs = off;
+    off += al(sizeof(Run) * (size_t)nruns);
     L.total = off;
     return L;
 }
@@ -243,6 +288,8 @@ struct sl_batch {
     int *items;
     unsigned *counters;
     double *tgrid;
+    int nruns;
+    Run *runs;           // the tiles in runs of up to RUN_TILES of one grid
     std::vector<double> t_host, dt_host;
     std::vector<int> dcur0;           // displacement buffer each grid's advect writes at a call start
     unsigned long long launches = 0;  // kernels launched by this batch's calls
@@ -268,16 +315,17 @@ static int batch_cfg(sl_grid *const *grids, int tile_config)
 extern "C" size_t sl_batch_workspace_bytes(sl_grid *const *grids, int count, int tile_config)
 {
     if (!grids || count < 1 || tile_config < 0 || tile_config > 5) return 0;
-    long long nitems = 0;
+    long long nitems = 0, nruns = 0;
     for (int q = 0; q < count; ++q) {
         if (!batch_eligible(grids[q])) return 0;
         if ((grids[q]->desc.max_order == 2) != (grids[0]->desc.max_order == 2)) return 0;
         int tx, ty;
         tile_counts(batch_cfg(grids, tile_config), grids[q], &tx, &ty);
         nitems += (long long)tx * ty;
+        nruns += ((long long)tx * ty + RUN_TILES - 1) / RUN_TILES;
     }
     if (nitems > (1LL << 30)) return 0;
-    return batch_layout(count, (int)nitems).total;
+    return batch_layout(count, (int)nitems, (int)nruns).total;
 }
 
 extern "C" sl_status sl_batch_create(sl_grid *const *grids, int count, void *const *const *fields,
@@ -332,15 +380,22 @@ extern "C" sl_status sl_batch_create(sl_grid *const *grids, int count, void *con
         tile_counts(b->cfg, g, &tx, &ty);
         e.tiles_x = tx;
         e.tile_base = (int)items.size();
+        e.ntiles = tx * ty;
         for (int t = 0; t < tx * ty; ++t) items.push_back(q);
     }
     b->nitems = (int)items.size();
-    b->L = batch_layout(count, b->nitems);
+    std::vector<Run> runs;
+    for (int q = 0; q < count; ++q)
+        for (int t = 0; t < table[q].ntiles; t += RUN_TILES)
+            runs.push_back({q, t, std::min(RUN_TILES, table[q].ntiles - t)});
+    b->nruns = (int)runs.size();
+    b->L = batch_layout(count, b->nitems, b->nruns);
     b->ws = (char *)dev_workspace;
     b->table = (BatchGrid *)(b->ws + b->L.table);
     b->items = (int *)(b->ws + b->L.items);
     b->counters = (unsigned *)(b->ws + b->L.counters);
     b->tgrid = (double *)(b->ws + b->L.tgrid);
+    b->runs = (Run *)(b->ws + b->L.runs);
     b->t_host.assign(t0, t0 + count);
     for (int q = 0; q < count; ++q) b->dcur0.push_back(grids[q]->dcur);
     b->dt_host.assign(dt, dt + count);
@@ -349,6 +404,7 @@ extern "C" sl_status sl_batch_create(sl_grid *const *grids, int count, void *con
     if (e == cudaSuccess) e = cudaMemcpy(b->table, table.data(), sizeof(BatchGrid) * count, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->items, items.data(), sizeof(int) * items.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->tgrid, t0, sizeof(double) * count, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b->runs, runs.data(), sizeof(Run) * runs.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         delete b;
         return SL_ERR_CUDA;
@@ -371,11 +427,11 @@ static cudaError_t launch_batch_seq(sl_batch *b, int nsteps, cudaStream_t s)
     const int simple = b->num_sms * 8;
     e = cudaMemsetAsync(b->counters, 0, sizeof(unsigned) * (SL_BATCH_MAX_STEPS + 2), s);
     if (e != cudaSuccess) return e;
-    batch_advect_kernel<Cfg><<<simple, Cfg::NT, 0, s>>>(b->table, b->items, b->nitems, b->counters + 0, b->tgrid);
+    batch_advect_kernel<Cfg><<<simple, Cfg::NT, 0, s>>>(b->table, b->runs, b->nruns, b->counters + 0, b->tgrid);
     for (int k = 0; k < nsteps; ++k)
         batch_step_kernel<Cfg, NF><<<ctas, Cfg::NT, smem, s>>>(b->table, b->items, b->nitems, b->counters + 1 + k,
                                                                b->tgrid, k, k + 1 == nsteps);
-    batch_finish_kernel<Cfg><<<simple, Cfg::NT, 0, s>>>(b->table, b->items, b->nitems,
+    batch_finish_kernel<Cfg><<<simple, Cfg::NT, 0, s>>>(b->table, b->runs, b->nruns,
                                                         b->counters + 1 + SL_BATCH_MAX_STEPS, b->tgrid, b->count,
                                                         nsteps);
     return cudaGetLastError();
@@ -398,11 +454,11 @@ static cudaError_t launch_batch_seq_z2(sl_batch *b, int nsteps, cudaStream_t s)
     e = cudaMemsetAsync(b->counters, 0, sizeof(unsigned) * (SL_BATCH_MAX_STEPS + 2), s);
     if (e != cudaSuccess) return e;
     // the quintic tiles have the 32 x 32 geometry of CfgA, whose trajectory and finishing kernels serve
-    batch_advect_kernel<CfgA><<<simple, CfgA::NT, 0, s>>>(b->table, b->items, b->nitems, b->counters + 0, b->tgrid);
+    batch_advect_kernel<CfgA><<<simple, CfgA::NT, 0, s>>>(b->table, b->runs, b->nruns, b->counters + 0, b->tgrid);
     for (int k = 0; k < nsteps; ++k)
         batch_step_z2_kernel<NF><<<ctas, CfgZ::NT, smem, s>>>(b->table, b->items, b->nitems, b->counters + 1 + k,
                                                               b->tgrid, k, k + 1 == nsteps);
-    batch_finish_kernel<CfgA><<<simple, CfgA::NT, 0, s>>>(b->table, b->items, b->nitems,
+    batch_finish_kernel<CfgA><<<simple, CfgA::NT, 0, s>>>(b->table, b->runs, b->nruns,
                                                           b->counters + 1 + SL_BATCH_MAX_STEPS, b->tgrid, b->count,
                                                           nsteps);
     return cudaGetLastError();

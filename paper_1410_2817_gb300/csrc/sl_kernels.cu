@@ -247,6 +247,29 @@ __global__ void __launch_bounds__(256) advect_kernel(GridArgs<T> g, VelArgs<T> v
     }
 }
 
+// The RK4 step of a 2-D Fourier velocity in FP32, two nodes a thread (rk4_fourier2d_pair): nodes i and
+// i + half of the grid.
+__global__ void __launch_bounds__(256, 3)
+    advect_fourier2d_kernel(GridArgs<float> g, VelArgs<float> v, float2 *__restrict__ D, unsigned half)
+{
+    __shared__ FourierPairs sf;
+    __shared__ float4 base[SL_PAIR_MODES][256];
+    sf.load(v, threadIdx.x);
+    __syncthreads();
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= half) return;
+    const unsigned j = i + half < g.N ? i + half : i;
+    int a[3], b[3];
+    node_coords<2>(i, g.n, a);
+    node_coords<2>(j, g.n, b);
+    const float2 X = make_float2(node_position(v.lo[0], a[0], v.dx[0]), node_position(v.lo[0], b[0], v.dx[0]));
+    const float2 Y = make_float2(node_position(v.lo[1], a[1], v.dx[1]), node_position(v.lo[1], b[1], v.dx[1]));
+    float2 Dx, Dy;
+    rk4_fourier2d_pair(sf, &base[0][threadIdx.x], 256, X, Y, Dx, Dy);
+    D[i] = make_float2(Dx.x, Dy.x);
+    if (j != i) D[j] = make_float2(Dx.y, Dy.y);
+}
+
 // The swirl's RK4 step in FP64 with as few FP64 instructions as the digits allow (110 per node for
 // offsets below 1/128 of the box, against 209 for rk4_trig_from; 1024^2: 410 -> 218 us, the FP64 pipe
 // busy 86 % of the time in both).  With S = sin(pi x), C = cos(pi x)
@@ -799,6 +822,13 @@ cudaError_t Launch<T>::advect(const sl_grid *g, void *D, double t, double dt, cu
                 w.By[q] = -b / g->dx[1];
             }
             advect_swirl64_kernel<<<blocks, 256, 0, s>>>(ga, va, w, (double2 *)D);
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (fourier2d_pairs(va)) {
+            const unsigned half = (unsigned)((g->N + 1) / 2);
+            advect_fourier2d_kernel<<<(half + 255) / 256, 256, 0, s>>>(ga, va, (float2 *)D, half);
             return cudaGetLastError();
         }
     }
