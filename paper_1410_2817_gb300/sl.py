@@ -126,10 +126,28 @@ def _check(status: int, where: str):
 
 def _stream(stream) -> C.c_void_p:
     if stream is None:
+        # the current stream's handle without building a Stream object (a microsecond a call)
+        if torch.cuda.is_initialized():
+            return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
         stream = torch.cuda.current_stream()
     if isinstance(stream, torch.cuda.Stream):
         return C.c_void_p(stream.cuda_stream)
     return C.c_void_p(int(stream))
+
+
+def _plane_array(ts):
+    """The host array of plane pointers alone: what a call passes (ctypes takes an array where a pointer
+    is expected; the cast of _planes, needed to store the pointer, costs a microsecond)."""
+    if isinstance(ts, torch.Tensor):
+        if not ts.is_cuda or not ts.is_contiguous() or ts.dim() < 2:
+            raise ValueError("field planes must be contiguous CUDA tensors")
+        nplanes = ts.shape[0]
+        base = ts.data_ptr()
+        if nplanes == 1:
+            return (C.c_void_p * 1)(base)
+        step = (ts.numel() // max(nplanes, 1)) * ts.element_size()
+        return (C.c_void_p * nplanes)(*[base + q * step for q in range(nplanes)])
+    return _planes(ts)[1]
 
 
 def _planes(ts):
@@ -208,9 +226,7 @@ def sl_advect_nodes_carried(h, fields: Sequence[torch.Tensor], dt: float, stream
 
 
 def sl_remap_fields(h, fin: Sequence[torch.Tensor], fout: Sequence[torch.Tensor], stream=None):
-    pi, _a = _planes(fin)
-    po, _b = _planes(fout)
-    _check(lib().sl_remap_fields(h, pi, po, _stream(stream)), "sl_remap_fields")
+    _check(lib().sl_remap_fields(h, _plane_array(fin), _plane_array(fout), _stream(stream)), "sl_remap_fields")
 
 
 def sl_remap_fields_debug(h, fin, fout, cell=None, xi=None, order=None, status=None, stream=None):
@@ -223,16 +239,14 @@ def sl_remap_fields_debug(h, fin, fout, cell=None, xi=None, order=None, status=N
 
 
 def sl_step(h, fields, scratch, t0: float, dt: float, nsteps: int, stream=None):
-    pf, _a = _planes(fields)
-    ps, _b = _planes(scratch)
-    _check(lib().sl_step(h, pf, ps, float(t0), float(dt), int(nsteps), _stream(stream)), "sl_step")
+    _check(lib().sl_step(h, _plane_array(fields), _plane_array(scratch), float(t0), float(dt), int(nsteps),
+                         _stream(stream)), "sl_step")
 
 
 def sl_step_out(h, fin, fout, scratch, t0: float, dt: float, nsteps: int, stream=None):
-    pi, _a = _planes(fin)
-    po, _b = _planes(fout)
-    ps, _c = _planes(scratch) if scratch is not None else (None, None)
-    _check(lib().sl_step_out(h, pi, po, ps, float(t0), float(dt), int(nsteps), _stream(stream)), "sl_step_out")
+    _check(lib().sl_step_out(h, _plane_array(fin), _plane_array(fout),
+                             None if scratch is None else _plane_array(scratch), float(t0), float(dt), int(nsteps),
+                             _stream(stream)), "sl_step_out")
 
 
 def sl_moments(h, field: torch.Tensor, pmax: int = 4, stream=None):
@@ -326,8 +340,12 @@ class Grid:
 
     def _fit(self, planes):
         """The nfields planes of this grid (a stacked tensor or a sequence); others raise."""
-        n = planes.shape[0] if isinstance(planes, torch.Tensor) else len(planes)
-        size = planes[0].numel() if n > 0 else 0
+        if isinstance(planes, torch.Tensor):  # (no per-plane view)
+            n = planes.shape[0]
+            size = planes.numel() // n if n > 0 else 0
+        else:
+            n = len(planes)
+            size = planes[0].numel() if n > 0 else 0
         if n != self.nfields or size != self.nnodes:
             raise ValueError(f"expected {self.nfields} planes of {self.nnodes} values")
         return planes
