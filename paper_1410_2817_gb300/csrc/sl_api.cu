@@ -117,12 +117,32 @@ struct Layout {
     size_t counters, stripes, sync, trig, partials, moment_out, flags, flags2, D0, D1, rk, rec, total;
 };
 
-// Does the grid run the two-phase 2-D FP32 step (whose records the workspace holds)?
+// Which calls of a 2-D FP32 grid the two-phase step serves, by its size counted in the 32 x 32 tiles of the
+// tiled kernel, of which 3 x 152 run in one wave.  `moving`: the launch also integrates the next step's
+// trajectories or takes them from the remapped fields.  Measured with warm L2, us a launch, two-phase /
+// tiled:
+//   up to 3 fields  256^2 (64 tiles) 7.8 / 10.7, 400^2 (169) 11.2 / 10.8, 513^2 (289) 13.1 / 11.5,
+//                   724^2 (529) 17.5 / 19.7, 1024^2 26.9 / 31.5, 2048^2 98.5 / 129: below a quarter of
+//                   a wave and above a whole one, and always for moving steps (their trajectories fill the
+//                   two-phase kernel's wait: 400^2 13.8 / 15.2, 513^2 16.3 / 16.6; Burgers 400^2 11.5 /
+//                   11.6, 513^2 13.1 / 13.7);
+//   4 fields        (two records a tap) 256^2 9.5 / 11.3, 400^2 13.7 / 11.5, 1024^2 36.3 / 33.6,
+//                   1449^2 (2116) 68.0 / 63.2, 2048^2 (4096) 129 / 139: small and large grids only.
+bool two_phase_size(const sl_grid_desc *d, bool moving)
+{
+    const long long tiles = ((d->n[0] + 31) / 32) * ((d->n[1] + 31) / 32), wave = 456;
+    if (d->nfields <= 3) return moving || tiles <= wave / 4 || tiles > wave;
+    return tiles <= wave / 5 || tiles > 7 * wave;
+}
+
+// Does the grid run the two-phase 2-D FP32 step on some call (its workspace then holds the records)?
 static bool has_records(const sl_grid_desc *d)
 {
+    const bool steady = d->velocity_kind != SL_VEL_SWIRL2D && d->velocity_kind != SL_VEL_CARRIED;
     return d->dim == 2 && d->dtype == SL_F32 && d->max_order <= 1 && d->nfields <= 4 && d->newton_mode == SL_NEWTON_MIXED &&
            d->walk_start == SL_START_BACKWARD && d->kernel != SL_KERNEL_GENERIC && d->tile_config == 0 &&
-           (d->n[0] + 3) * (d->n[1] + 3) < (1LL << 31);  // 32-bit record indices
+           (d->n[0] + 3) * (d->n[1] + 3) < (1LL << 31) &&  // 32-bit record indices
+           two_phase_size(d, !steady);
 }
 
 static Layout layout_of(const sl_grid_desc *d)
@@ -237,7 +257,8 @@ extern "C" sl_status sl_create_grid(const sl_grid_desc *desc, void *dev_workspac
     g->next_valid = 0;
     cudaError_t e = cudaGetDevice(&g->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->num_sms, cudaDevAttrMultiProcessorCount, g->device);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g->ws, 0, L.total, 0);
+    // (the records are written before they are read in every launch)
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->ws, 0, L.rec, 0);
     if (e == cudaSuccess) e = launch_trig_tables(g, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {

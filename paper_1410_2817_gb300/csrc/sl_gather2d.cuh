@@ -18,7 +18,7 @@
 // barriers per tile.  Back to back with warm L2 (us a launch; TMA-staged tiles / per-element-copy
 // tiles / this kernel), three fields of the swirl: remap 256^2 14.9 / 10.7 / 7.8, 1024^2 37.5 / 31.5 /
 // 26.9, 2048^2 124 / 129 / 98.5; fused step 1024^2 50.3 / 44.3 / 38.7; Burgers 1024^2 33.9 (tiles) / 28.3.
-// Where the tiles are better (sl_tiled.cu has the rule) they stay.
+// Where the tiles are better (two_phase_size has the rule) they stay.
 #pragma once
 
 #include "sl_tile2d.cuh"

@@ -109,6 +109,7 @@ size_t tiled2d_smem_bytes_cfgd(int nfields);
 double nlsw_viscosity(const sl_grid *g);
 int nlsw_kernels_per_step(const sl_grid *g);
 // 2-D FP32 step in two phases over flagged records (sl_gather2d.cu): tile configuration 0
+bool two_phase_size(const sl_grid_desc *d, bool moving);  // sl_api.cu
 size_t gather2d_record_bytes(long long n0, long long n1, int nfields);
 cudaError_t launch_gather2d(const sl_grid *g, const void *D, void *D_next, double t_next, double dt, bool fused,
                             const void *const *in, void *const *out, cudaStream_t s);

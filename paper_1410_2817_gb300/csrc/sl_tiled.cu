@@ -1,5 +1,5 @@
 // sl_tiled.cu -- dispatch of the FP32 production kernels: 2-D grids go to the two-phase kernel
-// (sl_gather2d.cuh; tile configuration 0, where use_gather says), to the persistent kernel with
+// (sl_gather2d.cuh; tile configuration 0, where two_phase_size says), to the persistent kernel with
 // TMA-staged windows (sl_remap2d.cuh; tile configurations 6 and 7, up to 3 fields, analytic
 // velocities) or to the shared-memory tiled kernels (sl_tile2d.cuh, one translation unit per tile
 // configuration; the quintic Z-spline to sl_tiled_z2.cu), 3-D grids to the staged or blocked
@@ -29,21 +29,10 @@ bool Launch<T>::tiled_supported(const sl_grid *g)
     return smem <= 200 * 1024;
 }
 
-// Does the two-phase kernel serve this call?  Counted in 32 x 32 tiles of the tiled kernel, whose 3 CTAs
-// per SM take up to 456 in one wave.  Measured with warm L2, us a launch, two-phase / tiled:
-//   up to 3 fields  256^2 (64 tiles) 7.8 / 10.7, 400^2 (169) 11.2 / 10.8, 513^2 (289) 13.1 / 11.5,
-//                   724^2 (529) 17.5 / 19.7, 1024^2 26.9 / 31.5, 2048^2 98.5 / 129: below a fifth of a
-//                   wave and above a whole one, and always where the launch also integrates
-//                   trajectories (which fill the two-phase kernel's wait: 400^2 13.8 / 15.2, 513^2
-//                   16.3 / 16.6) or is a carried step (400^2 11.5 / 11.6, 513^2 13.1 / 13.7);
-//   4 fields        (two records a tap) 256^2 9.5 / 11.3, 400^2 13.7 / 11.5, 1024^2 36.3 / 33.6,
-//                   1449^2 (2116) 68.0 / 63.2, 2048^2 (4096) 129 / 139: small and large grids only.
+// Does the two-phase kernel serve this call?
 static bool use_gather(const sl_grid *g, const void *D_next)
 {
-    if (g->rec == nullptr) return false;
-    const long long tiles = ((g->n[0] + 31) / 32) * ((g->n[1] + 31) / 32), wave = 3LL * g->num_sms;
-    if (g->nfields <= 3) return D_next != nullptr || tiles <= wave / 4 || tiles > wave;
-    return tiles <= wave / 5 || tiles > 7 * wave;
+    return g->rec != nullptr && two_phase_size(&g->desc, D_next != nullptr);
 }
 
 static cudaError_t launch_tiled2d(const sl_grid *g, const void *D, void *D_next, double t_next, double dt, bool fused,
