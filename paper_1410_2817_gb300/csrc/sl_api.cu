@@ -145,6 +145,14 @@ static bool has_records(const sl_grid_desc *d)
            two_phase_size(d, !steady);
 }
 
+// Do the grid's 3-D FP32 taps come from records?  (tile configuration 1 asks for the planes.)
+static bool has_records3(const sl_grid_desc *d)
+{
+    return d->dim == 3 && d->dtype == SL_F32 && d->max_order <= 1 && d->nfields <= 4 && d->newton_mode == SL_NEWTON_MIXED &&
+           d->walk_start == SL_START_BACKWARD && d->kernel != SL_KERNEL_GENERIC && d->tile_config != 1 &&
+           (d->n[0] + 3) * (d->n[1] + 3) * (d->n[2] + 3) < (1LL << 31);  // 32-bit record indices
+}
+
 static Layout layout_of(const sl_grid_desc *d)
 {
     Layout L;
@@ -182,6 +190,7 @@ static Layout layout_of(const sl_grid_desc *d)
     L.rk = off;
     if (d->velocity_kind == SL_VEL_NLSW) off += align256((size_t)N * 13 * ts);
     L.rec = off;
+    if (has_records3(d)) off += record3d_bytes(d);
     if (has_records(d)) off += gather2d_record_bytes(d->n[0], d->n[1], d->nfields);
     L.total = off;
     return L;
@@ -241,7 +250,7 @@ extern "C" sl_status sl_create_grid(const sl_grid_desc *desc, void *dev_workspac
     g->moment_out = (double *)(g->ws + L.moment_out);
     g->flags = (uint8_t *)(g->ws + L.flags);
     g->flags2 = (uint8_t *)(g->ws + L.flags2);
-    g->rec = has_records(desc) ? (void *)(g->ws + L.rec) : nullptr;
+    g->rec = has_records(desc) || has_records3(desc) ? (void *)(g->ws + L.rec) : nullptr;
     g->sync = (unsigned *)(g->ws + L.sync);
     g->D[0] = g->ws + L.D0;
     g->D[1] = g->ws + L.D1;

@@ -6,6 +6,13 @@
 //   * remap_blocked3d_kernel: one thread per target; a CTA covers a 16x4x4 block of targets so
 //     that the element search (Sec. 2.2, Newton in FP32 with FP64 re-solves near faces) and the
 //     64-tap tricubic sums (eq. multiZ) of neighbouring targets hit the same L1 lines;
+//     Grids of up to four fields read their taps from records (the fields of a node side by side, with
+//     the periodic images a stencil may reach, written by the flag pass): one load a tap at a fixed
+//     offset instead of one a field and tap at a computed address.  Bound by instruction issue (69 %
+//     active at 256^3): the 256^3 x 2 fused launch 1260 -> 1045 us, the flag pass 117 -> 179 us for
+//     the 134 MB of records it writes, the step 1338 -> 1174 us; 79^3 x 3 remap 69.5 -> 53.2 us;
+//     192^3 step, warm, 1 / 2 / 3 / 4 fields 467 / 509 / 781 / 833 -> 374 / 440 / 581 / 614 us, 32^3
+//     about equal;
 //   * remap_staged3d_kernel (plain remaps of up to 2 fields): the same blocks and element search,
 //     with the field values of the block's stencils copied to shared memory (TMA boxes inside the
 //     grid, per-element copies across the periodic seam) while the search runs, and the tap sums
@@ -50,9 +57,40 @@ struct Fields3 {
 // are 32 x 8 threads over (x, y) and loop over y and z, so no index is divided.
 constexpr int FX = 29;  // nodes written per warp and row by flags_x3d
 
+// Records of a grid: float, float2 or float4 per node for 1, 2, 3-4 fields, rows of n0 + 3 and planes of
+// n1 + 3 rows: one image node below and two above along every axis.
+constexpr int R3_LO = 1, R3_HI = 2, R3_PAD = 3;
+__host__ __device__ constexpr int rec3_width(int nf) { return nf <= 2 ? nf : 4; }
+
+template <int NFM>
+__device__ __forceinline__ void store_rec3(float *rec, int width, unsigned i, const float h[NFM])
+{
+    if (NFM == 4)
+        reinterpret_cast<float4 *>(rec)[i] = make_float4(h[0], h[1], h[NFM > 2 ? 2 : 0], h[NFM > 3 ? 3 : 0]);
+    else if (width == 2)
+        reinterpret_cast<float2 *>(rec)[i] = make_float2(h[0], h[1]);
+    else
+        rec[i] = h[0];
+}
+// the periodic images of the node with record i: wx, wy, wz are what an image is shifted by (0: none)
+template <int NFM>
+__device__ __noinline__ void store_images3(float *rec, int width, unsigned i, int wx, int wy, int wz, float h0, float h1,
+                                           float h2, float h3)
+{
+    const float all[4] = {h0, h1, h2, h3};
+    float h[NFM];
+#pragma unroll
+    for (int q = 0; q < NFM; ++q) h[q] = all[q];
+#pragma unroll 1
+    for (int m = 1; m < 8; ++m) {
+        if (((m & 1) && wx == 0) || ((m & 2) && wy == 0) || ((m & 4) && wz == 0)) continue;
+        store_rec3<NFM>(rec, width, i + (unsigned)((m & 1 ? wx : 0) + (m & 2 ? wy : 0) + (m & 4 ? wz : 0)), h);
+    }
+}
+
 template <int NFM>
 __global__ void __launch_bounds__(256)
-    flags_x3d_kernel(Geo3 g, int nfields, float thr, Fields3 f, uint8_t *out, int zchunk)
+    flags_x3d_kernel(Geo3 g, int nfields, float thr, Fields3 f, uint8_t *out, int zchunk, float *rec)
 {
     const int lane = threadIdx.x;
     const int x0 = blockIdx.x * FX;
@@ -64,6 +102,12 @@ __global__ void __launch_bounds__(256)
         const long long yc = (long long)y * g.n0 + x, ym = (long long)wrap_near(y - 1, g.n1) * g.n0 + x,
                         yp = (long long)wrap_near(y + 1, g.n1) * g.n0 + x;
         const long long xl = (long long)y * g.n0 + xm, xr = (long long)y * g.n0 + xp;
+        // the node's record in plane 0 and the shifts of its images along x and y, in records
+        const int p0 = g.n0 + R3_PAD, p01 = p0 * (g.n1 + R3_PAD), xn = x0 - 1 + lane;
+        const bool put = NFM <= 4 && rec != nullptr && lane >= 1 && lane <= FX && xn < g.n0;
+        const unsigned ri = (unsigned)(p01 + (y + R3_LO) * p0 + xn + R3_LO);
+        const int wx = xn < R3_HI ? g.n0 : (xn >= g.n0 - R3_LO ? -g.n0 : 0);
+        const int wy = y < R3_HI ? g.n1 * p0 : (y >= g.n1 - R3_LO ? -g.n1 * p0 : 0);
         // a thread walks z through its chunk keeping the centre values of planes z-1 and z
         float cm[NFM], cc[NFM];
 #pragma unroll
@@ -78,6 +122,16 @@ __global__ void __launch_bounds__(256)
         for (int z = zb; z < ze; ++z) {
             const long long zc = z * plane, zp = wrap_near(z + 1, g.n2) * plane;
             unsigned bits = 0;
+            if (put) {
+                constexpr int M = NFM <= 4 ? NFM : 4;
+                const unsigned i = ri + (unsigned)(z * p01);
+                const int width = rec3_width(nfields);
+                store_rec3<M>(rec, width, i, cc);
+                const int wz = z < R3_HI ? g.n2 * p01 : (z >= g.n2 - R3_LO ? -g.n2 * p01 : 0);
+                if ((wx | wy | wz) != 0)
+                    store_images3<M>(rec, width, i, wx, wy, wz, cc[0], cc[1], NFM > 2 ? cc[NFM > 2 ? 2 : 0] : 0.f,
+                                     NFM > 3 ? cc[NFM > 3 ? 3 : 0] : 0.f);
+            }
 #pragma unroll
             for (int q = 0; q < NFM; ++q) {
                 if (q < nfields) {
@@ -257,6 +311,7 @@ struct Blocked3Args {
     const uint8_t *box;   // OR of the flags over each element's 4x4x4 stencil
     Fields3 f;
     DevCounters *counters;  // the grid's SL_COUNTER_STRIPES per-SM copies of its counters
+    const float *rec;       // records (null: the taps are gathered from the planes)
 };
 
 // The 4x4x4 stencil taps of element c from global memory: node offsets along each axis (direct when
@@ -356,6 +411,95 @@ __device__ __forceinline__ void tap_sums(const Taps &tp, int nfields, const floa
     }
 }
 
+// The same sums from the records, W = 1, 2, 4 fields a load, for the 4x4x4 taps starting at record o; the
+// trilinear ones only where a lane of the warp has a flagged field (bits).
+template <int W>
+struct Rec3;
+template <>
+struct Rec3<1> {
+    typedef float T;
+    static __device__ __forceinline__ float2 pair(float t, int) { return make_float2(t, t); }
+};
+template <>
+struct Rec3<2> {
+    typedef float2 T;
+    static __device__ __forceinline__ float2 pair(float2 t, int) { return t; }
+};
+template <>
+struct Rec3<4> {
+    typedef float4 T;
+    static __device__ __forceinline__ float2 pair(const float4 &t, int p)
+    {
+        return p == 0 ? make_float2(t.x, t.y) : make_float2(t.z, t.w);
+    }
+};
+
+template <int W>
+__device__ __forceinline__ void record_sums(const float *rec, unsigned o, int p0, unsigned p01, const float wc[3][4],
+                                            const float xf[3], unsigned bits, float v[W])
+{
+    typedef typename Rec3<W>::T T;
+    constexpr int NP = (W + 1) / 2;
+    const T *r0 = reinterpret_cast<const T *>(rec) + o;
+    float2 cs[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) cs[p] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int kz = 0; kz < 4; ++kz) {
+        float2 sy[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) sy[p] = make_float2(0.f, 0.f);
+        const T *r = r0 + (size_t)(unsigned)kz * p01;
+#pragma unroll
+        for (int ky = 0; ky < 4; ++ky) {
+            const T t0 = __ldg(r), t1 = __ldg(r + 1), t2 = __ldg(r + 2), t3 = __ldg(r + 3);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                float2 q = __fmul2_rn(make_float2(wc[0][0], wc[0][0]), Rec3<W>::pair(t0, p));
+                q = __ffma2_rn(make_float2(wc[0][1], wc[0][1]), Rec3<W>::pair(t1, p), q);
+                q = __ffma2_rn(make_float2(wc[0][2], wc[0][2]), Rec3<W>::pair(t2, p), q);
+                q = __ffma2_rn(make_float2(wc[0][3], wc[0][3]), Rec3<W>::pair(t3, p), q);
+                sy[p] = __ffma2_rn(make_float2(wc[1][ky], wc[1][ky]), q, sy[p]);
+            }
+            r += p0;
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) cs[p] = __ffma2_rn(make_float2(wc[2][kz], wc[2][kz]), sy[p], cs[p]);
+    }
+#pragma unroll
+    for (int c = 0; c < W; ++c) v[c] = (c & 1) ? cs[c / 2].y : cs[c / 2].x;
+    if (bits & ((1u << W) - 1u)) {
+        const T *r = r0 + p01 + p0 + 1;
+        float2 ls[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) ls[p] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int kz = 0; kz < 2; ++kz) {
+            float2 sy[NP];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) sy[p] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int ky = 0; ky < 2; ++ky) {
+                const T *q = r + (kz ? p01 : 0u) + (ky ? p0 : 0);
+                const T t1 = __ldg(q), t2 = __ldg(q + 1);
+                const float vy = ky == 0 ? 1.f - xf[1] : xf[1];
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+                    sy[p] = __ffma2_rn(make_float2(vy, vy),
+                                       __ffma2_rn(make_float2(xf[0], xf[0]), Rec3<W>::pair(t2, p),
+                                                  __fmul2_rn(make_float2(1.f - xf[0], 1.f - xf[0]), Rec3<W>::pair(t1, p))),
+                                       sy[p]);
+            }
+            const float vz = kz == 0 ? 1.f - xf[2] : xf[2];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) ls[p] = __ffma2_rn(make_float2(vz, vz), sy[p], ls[p]);
+        }
+#pragma unroll
+        for (int c = 0; c < W; ++c)
+            if ((bits >> c) & 1u) v[c] = (c & 1) ? ls[c / 2].y : ls[c / 2].x;
+    }
+}
+
 // Start element of a target: one fixed-point step s <- j - D(s) from s0 = j - D_j, with D(s0)
 // trilinear over the 8 nodes around s0 (the walk still decides); c keeps floor(s0) where the step
 // is not finite or moves by 4 cells or more.
@@ -397,7 +541,8 @@ __device__ __forceinline__ void start_point3(const int j[3], const float4 dj, fl
 
 // N64: every target's element search and Newton inversion in FP64 (SL_NEWTON_F64) from the refined
 // start; otherwise in FP32 with an FP64 re-solve of failed or near-degenerate targets.
-template <int NFM, bool FUSED, bool N64>
+// RW: fields a record holds (1, 2, 4), 0 without records.
+template <int NFM, bool FUSED, bool N64, int RW>
 __global__ void __launch_bounds__(NT3, 4) remap_blocked3d_kernel(const Blocked3Args a, const VelArgs<float> vn)
 {
     const Geo3 &g = a.g;
@@ -447,20 +592,40 @@ __global__ void __launch_bounds__(NT3, 4) remap_blocked3d_kernel(const Blocked3A
             float wc[3][4];
 #pragma unroll
             for (int q = 0; q < 3; ++q) cubic_w(xf[q], wc[q]);
-            const GlobalTaps3 tp(g, a.f, a.nfields, c);
-            unsigned bits = 0xffu;
-            if (a.max_order >= 1) bits = __ldg(a.box + (tp.oz[1] + tp.oy[1] + (unsigned)tp.ox[1]));
-            // one instance of the tap loop (a second one for stencils away from the x seam made
-            // the kernel larger and measured slower)
-            float cub[NFM], lin[NFM];
-            tap_sums<NFM>(tp, a.nfields, wc, xf, cub, lin);
+            if constexpr (RW > 0) {
+                const int wx = wrap3(c[0], g.n0), wy = wrap3(c[1], g.n1), wz = wrap3(c[2], g.n2);
+                unsigned bits = 0xffu;
+                if (a.max_order >= 1)
+                    bits = __ldg(a.box + (((unsigned)wz * (unsigned)g.n1 + (unsigned)wy) * (unsigned)g.n0 + (unsigned)wx));
+                const int p0 = g.n0 + R3_PAD;
+                const unsigned p01 = (unsigned)p0 * (unsigned)(g.n1 + R3_PAD);
+                float v[RW];
+                // record (wx - 1, wy - 1, wz - 1): the image margin below is one node
+                record_sums<RW>(a.rec, (unsigned)wz * p01 + (unsigned)wy * (unsigned)p0 + (unsigned)wx, p0, p01, wc, xf, bits, v);
 #pragma unroll
-            for (int q = 0; q < NFM; ++q) {
-                if (q >= a.nfields) break;
-                const bool useL = ((bits >> q) & 1u) != 0u;
-                cnt.oh0 += useL;
-                cnt.oh1 += !useL;
-                a.f.out[q][jj] = useL ? lin[q] : cub[q];
+                for (int q = 0; q < RW; ++q) {
+                    if (q >= a.nfields) break;
+                    const bool useL = ((bits >> q) & 1u) != 0u;
+                    cnt.oh0 += useL;
+                    cnt.oh1 += !useL;
+                    a.f.out[q][jj] = v[q];
+                }
+            } else {
+                const GlobalTaps3 tp(g, a.f, a.nfields, c);
+                unsigned bits = 0xffu;
+                if (a.max_order >= 1) bits = __ldg(a.box + (tp.oz[1] + tp.oy[1] + (unsigned)tp.ox[1]));
+                // one instance of the tap loop (a second one for stencils away from the x seam made
+                // the kernel larger and measured slower)
+                float cub[NFM], lin[NFM];
+                tap_sums<NFM>(tp, a.nfields, wc, xf, cub, lin);
+#pragma unroll
+                for (int q = 0; q < NFM; ++q) {
+                    if (q >= a.nfields) break;
+                    const bool useL = ((bits >> q) & 1u) != 0u;
+                    cnt.oh0 += useL;
+                    cnt.oh1 += !useL;
+                    a.f.out[q][jj] = useL ? lin[q] : cub[q];
+                }
             }
         }
         if (FUSED && a.D_next != nullptr) {
@@ -740,8 +905,24 @@ __global__ void __launch_bounds__(NT3, 4)
 
 }  // namespace
 
+// The staged kernel serves plain remaps of FP32 grids with up to 2 fields whose targets invert in
+// FP32 (FP64 re-solves only for failed or degenerate ones), unless tile configuration 1 asks for
+// the L1 path.
+static bool staged3d_supported(const sl_grid *g)
+{
+    return g->nfields <= 2 && g->desc.newton_mode != SL_NEWTON_F64 && g->desc.tile_config != 1;
+}
+
+// bytes of a 3-D grid's records
+size_t record3d_bytes(const sl_grid_desc *d)
+{
+    return (size_t)(d->n[0] + R3_PAD) * (size_t)(d->n[1] + R3_PAD) * (size_t)(d->n[2] + R3_PAD) * 4 *
+           (size_t)rec3_width(d->nfields);
+}
+
 // box flags of a 3-D FP32 grid: flags ORed along x into `flags`, then over y and z into `tmp`
-cudaError_t launch_box_flags3d(const sl_grid *g, const void *const *in, uint8_t *flags, uint8_t *tmp, cudaStream_t s)
+cudaError_t launch_box_flags3d(const sl_grid *g, const void *const *in, uint8_t *flags, uint8_t *tmp, bool fused,
+                               cudaStream_t s)
 {
     Geo3 geo = {(int)g->n[0], (int)g->n[1], (int)g->n[2]};
     Fields3 f;
@@ -750,15 +931,21 @@ cudaError_t launch_box_flags3d(const sl_grid *g, const void *const *in, uint8_t 
     const dim3 block(32, 8);
     const unsigned gy = (unsigned)std::min<long long>((g->n[1] + 7) / 8, 65535);
     const unsigned gz = (unsigned)std::min<long long>(g->n[2], 65535);
-    const int zchunk = (int)std::max<long long>(16, (g->n[2] + 65534) / 65535);
+    // planes a thread walks: 16, or 4 where that leaves the SMs short of blocks (79^3 x 3: 150 blocks of 16
+    // planes, each a chain of 16 loads, 27.8 us; 13.9 us with 4)
+    const long long cols = (long long)((g->n[0] + FX - 1) / FX) * gy;
+    const int zwalk = cols * ((g->n[2] + 15) / 16) >= 8LL * g->num_sms ? 16 : 4;
+    const int zchunk = (int)std::max<long long>(zwalk, (g->n[2] + 65534) / 65535);
     const dim3 gridf((unsigned)((g->n[0] + FX - 1) / FX), gy, (unsigned)((g->n[2] + zchunk - 1) / zchunk));
     const float thr = (float)g->desc.limiter_threshold;
+    // (a plain remap on the staged kernel reads the planes)
+    float *rec = !fused && staged3d_supported(g) ? nullptr : (float *)g->rec;
     if (g->nfields <= 2)
-        flags_x3d_kernel<2><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk);
+        flags_x3d_kernel<2><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk, rec);
     else if (g->nfields <= 4)
-        flags_x3d_kernel<4><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk);
+        flags_x3d_kernel<4><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk, rec);
     else
-        flags_x3d_kernel<8><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk);
+        flags_x3d_kernel<8><<<gridf, block, 0, s>>>(geo, g->nfields, thr, f, flags, zchunk, nullptr);
     // the byte buffers start 256-byte aligned; rows of a multiple of 4 nodes keep 32-bit alignment
     if (g->n[0] % 4 == 0) {
         const dim3 gridb((unsigned)((g->n[0] / 4 + 31) / 32), gy, gz);
@@ -774,22 +961,23 @@ template <bool N64>
 static void launch_b3(int nfm, bool fused, dim3 grid, cudaStream_t s, const Blocked3Args &a, const VelArgs<float> &vn)
 {
     if (fused) {
-        if (nfm == 2) remap_blocked3d_kernel<2, true, N64><<<grid, NT3, 0, s>>>(a, vn);
-        else if (nfm == 4) remap_blocked3d_kernel<4, true, N64><<<grid, NT3, 0, s>>>(a, vn);
-        else remap_blocked3d_kernel<8, true, N64><<<grid, NT3, 0, s>>>(a, vn);
+        if (nfm == 2) remap_blocked3d_kernel<2, true, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
+        else if (nfm == 4) remap_blocked3d_kernel<4, true, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
+        else remap_blocked3d_kernel<8, true, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
     } else {
-        if (nfm == 2) remap_blocked3d_kernel<2, false, N64><<<grid, NT3, 0, s>>>(a, vn);
-        else if (nfm == 4) remap_blocked3d_kernel<4, false, N64><<<grid, NT3, 0, s>>>(a, vn);
-        else remap_blocked3d_kernel<8, false, N64><<<grid, NT3, 0, s>>>(a, vn);
+        if (nfm == 2) remap_blocked3d_kernel<2, false, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
+        else if (nfm == 4) remap_blocked3d_kernel<4, false, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
+        else remap_blocked3d_kernel<8, false, N64, 0><<<grid, NT3, 0, s>>>(a, vn);
     }
 }
 
-// The staged kernel serves plain remaps of FP32 grids with up to 2 fields whose targets invert in
-// FP32 (FP64 re-solves only for failed or degenerate ones), unless tile configuration 1 asks for
-// the L1 path.
-static bool staged3d_supported(const sl_grid *g)
+template <int RW>
+static void launch_r3(bool fused, dim3 grid, cudaStream_t s, const Blocked3Args &a, const VelArgs<float> &vn)
 {
-    return g->nfields <= 2 && g->desc.newton_mode != SL_NEWTON_F64 && g->desc.tile_config != 1;
+    if (fused)
+        remap_blocked3d_kernel<RW == 1 ? 2 : RW, true, false, RW><<<grid, NT3, 0, s>>>(a, vn);
+    else
+        remap_blocked3d_kernel<RW == 1 ? 2 : RW, false, false, RW><<<grid, NT3, 0, s>>>(a, vn);
 }
 
 template <int NF>
@@ -851,6 +1039,17 @@ cudaError_t launch_blocked3d(const sl_grid *g, const void *D, void *D_next, cons
     // integrates the next trajectories, measured faster on the blocked kernel)
     if (!fused && staged3d_supported(g)) return launch_staged3d(g, a, grid, s);
     const int nfm = g->nfields <= 2 ? 2 : g->nfields <= 4 ? 4 : 8;
+    a.rec = (const float *)g->rec;
+    if (a.rec != nullptr) {
+        const int w = rec3_width(g->nfields);
+        if (w == 1)
+            launch_r3<1>(fused, grid, s, a, vn);
+        else if (w == 2)
+            launch_r3<2>(fused, grid, s, a, vn);
+        else
+            launch_r3<4>(fused, grid, s, a, vn);
+        return cudaGetLastError();
+    }
     if (g->desc.newton_mode == SL_NEWTON_F64)
         launch_b3<true>(nfm, fused, grid, s, a, vn);
     else

@@ -27,7 +27,8 @@ struct sl_grid {
     double *moment_out;          // 8 doubles
     uint8_t *flags;              // N
     uint8_t *flags2;             // N (second byte buffer: separable OR of flags over stencils)
-    void *rec;                   // records of the two-phase 2-D FP32 step (null where it does not run)
+    void *rec;                   // records of the two-phase 2-D FP32 step or of the 3-D FP32 taps (null
+                                 // where the grid's calls read the planes)
     unsigned *sync;              // its phase counters (zero between launches)
     void *D[2];                  // two displacement buffers (ping-pong for the pipelined step)
     int dcur;                    // index of the current displacement
@@ -83,7 +84,10 @@ struct Launch {
 // 3-D FP32 kernels (sl_blocked3d.cu): box flags end up in `tmp`; launch_blocked3d runs a plain
 // remap on the staged kernel where it applies, a fused step (and the rest) on the blocked one
 cudaError_t launch_trig_tables(const sl_grid *g, cudaStream_t s);
-cudaError_t launch_box_flags3d(const sl_grid *g, const void *const *in, uint8_t *flags, uint8_t *tmp, cudaStream_t s);
+// (and the records of the launch that follows: fused or plain)
+cudaError_t launch_box_flags3d(const sl_grid *g, const void *const *in, uint8_t *flags, uint8_t *tmp, bool fused,
+                               cudaStream_t s);
+size_t record3d_bytes(const sl_grid_desc *d);
 cudaError_t launch_blocked3d(const sl_grid *g, const void *D, void *D_next, const uint8_t *box, double t_next,
                              double dt, bool fused, const void *const *in, void *const *out, cudaStream_t s);
 // kernels one tiled remap / fused step call launches

@@ -60,7 +60,7 @@ cudaError_t Launch<T>::remap_tiled(const sl_grid *g, const void *D, const void *
 {
     if (!tiled_supported(g)) return cudaErrorNotSupported;
     if (g->dim == 3) {
-        cudaError_t e = launch_box_flags3d(g, in, g->flags, g->flags2, s);
+        cudaError_t e = launch_box_flags3d(g, in, g->flags, g->flags2, false, s);
         if (e != cudaSuccess) return e;
         return launch_blocked3d(g, D, nullptr, g->flags2, 0.0, 0.0, false, in, out, s);
     }
@@ -73,7 +73,7 @@ cudaError_t Launch<T>::step_fused(const sl_grid *g, const void *D, void *D_next,
 {
     if (!tiled_supported(g)) return cudaErrorNotSupported;
     if (g->dim == 3) {
-        cudaError_t e = launch_box_flags3d(g, in, g->flags, g->flags2, s);
+        cudaError_t e = launch_box_flags3d(g, in, g->flags, g->flags2, true, s);
         if (e != cudaSuccess) return e;
         return launch_blocked3d(g, D, D_next, g->flags2, t_next, dt, true, in, out, s);
     }
