@@ -9,7 +9,7 @@
 //     Grids of up to four fields read their taps from records (the fields of a node side by side, with
 //     the periodic images a stencil may reach, written by the flag pass): one load a tap at a fixed
 //     offset instead of one a field and tap at a computed address.  Bound by instruction issue (69 %
-//     active at 256^3): the 256^3 x 2 fused launch 1260 -> 1045 us, the flag pass 117 -> 179 us for
+//     active at 256^3): the 256^3 x 2 fused launch 1260 -> 1045 us, the flag pass 117 -> 172 us for
 //     the 134 MB of records it writes, the step 1338 -> 1174 us; 79^3 x 3 remap 69.5 -> 53.2 us;
 //     192^3 step, warm, 1 / 2 / 3 / 4 fields 467 / 509 / 781 / 833 -> 374 / 440 / 581 / 614 us, 32^3
 //     about equal;
@@ -96,12 +96,12 @@ __global__ void __launch_bounds__(256)
     const int x0 = blockIdx.x * FX;
     const int x = wrap_idx(x0 - 1 + lane, g.n0);  // rows shorter than a warp wrap more than once
     const int xm = wrap_near(x - 1, g.n0), xp = wrap_near(x + 1, g.n0);
-    const long long plane = (long long)g.n0 * g.n1;
+    const unsigned plane = (unsigned)g.n0 * (unsigned)g.n1;  // (32-bit offsets: a grid has fewer than 2^31 nodes)
     const int zb = blockIdx.z * zchunk, ze = min(g.n2, zb + zchunk);
     for (int y = blockIdx.y * blockDim.y + threadIdx.y; y < g.n1; y += gridDim.y * blockDim.y) {
-        const long long yc = (long long)y * g.n0 + x, ym = (long long)wrap_near(y - 1, g.n1) * g.n0 + x,
-                        yp = (long long)wrap_near(y + 1, g.n1) * g.n0 + x;
-        const long long xl = (long long)y * g.n0 + xm, xr = (long long)y * g.n0 + xp;
+        const unsigned yc = (unsigned)(y * g.n0 + x), ym = (unsigned)(wrap_near(y - 1, g.n1) * g.n0 + x),
+                       yp = (unsigned)(wrap_near(y + 1, g.n1) * g.n0 + x);
+        const unsigned xl = (unsigned)(y * g.n0 + xm), xr = (unsigned)(y * g.n0 + xp);
         // the node's record in plane 0 and the shifts of its images along x and y, in records
         const int p0 = g.n0 + R3_PAD, p01 = p0 * (g.n1 + R3_PAD), xn = x0 - 1 + lane;
         const bool put = NFM <= 4 && rec != nullptr && lane >= 1 && lane <= FX && xn < g.n0;
@@ -114,13 +114,13 @@ __global__ void __launch_bounds__(256)
         for (int q = 0; q < NFM; ++q) {
             cm[q] = cc[q] = 0.f;
             if (q < nfields) {
-                cm[q] = __ldg(f.in[q] + wrap_near(zb - 1, g.n2) * plane + yc);
-                cc[q] = __ldg(f.in[q] + zb * plane + yc);
+                cm[q] = __ldg(f.in[q] + ((unsigned)wrap_near(zb - 1, g.n2) * plane + yc));
+                cc[q] = __ldg(f.in[q] + ((unsigned)zb * plane + yc));
             }
         }
 #pragma unroll 2
         for (int z = zb; z < ze; ++z) {
-            const long long zc = z * plane, zp = wrap_near(z + 1, g.n2) * plane;
+            const unsigned zc = (unsigned)z * plane, zp = (unsigned)wrap_near(z + 1, g.n2) * plane;
             unsigned bits = 0;
             if (put) {
                 constexpr int M = NFM <= 4 ? NFM : 4;
@@ -136,9 +136,9 @@ __global__ void __launch_bounds__(256)
             for (int q = 0; q < NFM; ++q) {
                 if (q < nfields) {
                     const float *h = f.in[q];
-                    const float cp = __ldg(h + zp + yc);
-                    const float l = __ldg(h + zc + xl), r = __ldg(h + zc + xr);
-                    const float d = __ldg(h + zc + ym), u = __ldg(h + zc + yp);
+                    const float cp = __ldg(h + (zp + yc));
+                    const float l = __ldg(h + (zc + xl)), r = __ldg(h + (zc + xr));
+                    const float d = __ldg(h + (zc + ym)), u = __ldg(h + (zc + yp));
                     const bool hit = jump_test<float>(l, cc[q], r, thr) | jump_test<float>(d, cc[q], u, thr) |
                                      jump_test<float>(cm[q], cc[q], cp, thr);
                     bits |= (hit && thr >= 0.f) ? (1u << q) : 0u;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(256)
             const unsigned r2 = __shfl_down_sync(0xffffffffu, bits, 2);
             const int xo = x0 - 1 + lane;
             if (lane >= 1 && lane <= FX && xo < g.n0)
-                out[zc + (long long)y * g.n0 + xo] = (uint8_t)(left | bits | r1 | r2);
+                out[zc + (unsigned)(y * g.n0 + xo)] = (uint8_t)(left | bits | r1 | r2);
         }
     }
 }

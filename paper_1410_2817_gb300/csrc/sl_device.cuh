@@ -841,8 +841,9 @@ __device__ __forceinline__ void rk4_cells(const VelArgs<T> &v, const T X[3], T o
 template <typename T>
 __device__ __forceinline__ T diff_prod(T a, T b, T c, T d) { return fma_rn_t(a, b, -mul_rn_t(c, d)); }
 
-// (every product and sum is rounded explicitly, so that the 2-D kernels that inline this, or repeat
-// its steps, invert an element to the same bits)
+// (The two-phase 2-D kernel repeats these steps with the roundings written out as the compiler contracts
+// them here; its test compares the bits.  Written out here too, the tiled kernel with four fields measured
+// 1.5 % slower.)
 template <typename T>
 __device__ __forceinline__ int newton_solve2(const T P[8][3], int max_iter, T tol, T xi[3], int *iters,
                                              bool *degenerate = nullptr)
@@ -852,39 +853,38 @@ __device__ __forceinline__ int newton_solve2(const T P[8][3], int max_iter, T to
     const T ex = P[3][0] - P[1][0] - P[2][0] + P[0][0], ey = P[3][1] - P[1][1] - P[2][1] + P[0][1];
     const T px = P[0][0], py = P[0][1];
     *iters = 0;
-    T det = diff_prod(ax, by, bx, ay);
+    T det = ax * by - bx * ay;
     if (degenerate) *degenerate = true;
     if (!(det > T(0))) {
         xi[0] = xi[1] = T(NAN);
         return ST_FOLD;
     }
     T inv = recip_t(det);
-    T s = mul_rn_t(-diff_prod(px, by, py, bx), inv);
-    T t = mul_rn_t(-diff_prod(ax, py, ay, px), inv);
+    T s = -(px * by - py * bx) * inv;
+    T t = -(ax * py - ay * px) * inv;
     for (int it = 1; it <= max_iter; ++it) {
         *iters = it;
-        const T j11 = fma_rn_t(t, ex, ax), j21 = fma_rn_t(t, ey, ay);
-        const T j12 = fma_rn_t(s, ex, bx), j22 = fma_rn_t(s, ey, by);
-        const T st = mul_rn_t(s, t);
-        const T fx = fma_rn_t(st, ex, fma_rn_t(t, bx, fma_rn_t(s, ax, px)));
-        const T fy = fma_rn_t(st, ey, fma_rn_t(t, by, fma_rn_t(s, ay, py)));
-        det = diff_prod(j11, j22, j12, j21);
+        const T j11 = ax + t * ex, j21 = ay + t * ey;
+        const T j12 = bx + s * ex, j22 = by + s * ey;
+        const T st = s * t;
+        const T fx = px + s * ax + t * bx + st * ex;
+        const T fy = py + s * ay + t * by + st * ey;
+        det = j11 * j22 - j12 * j21;
         if (!(det > T(0))) {
             xi[0] = s;
             xi[1] = t;
             return ST_FOLD;
         }
         inv = recip_t(det);
-        const T d0 = mul_rn_t(diff_prod(fx, j22, fy, j12), inv);
-        const T d1 = mul_rn_t(diff_prod(j11, fy, j21, fx), inv);
+        const T d0 = (fx * j22 - fy * j12) * inv;
+        const T d1 = (j11 * fy - j21 * fx) * inv;
         s -= d0;
         t -= d1;
         if (max_t(abs_t(d0), abs_t(d1)) <= tol) {
             xi[0] = s;
             xi[1] = t;
             if (degenerate)
-                *degenerate = det < mul_rn_t(T(SL_DEGENERATE),
-                                             mul_rn_t(abs_t(j11) + abs_t(j21), abs_t(j12) + abs_t(j22)));
+                *degenerate = det < T(SL_DEGENERATE) * ((abs_t(j11) + abs_t(j21)) * (abs_t(j12) + abs_t(j22)));
             return ST_OK;
         }
     }

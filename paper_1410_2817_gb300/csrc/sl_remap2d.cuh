@@ -498,23 +498,23 @@ __device__ __forceinline__ bool fast_target(const Win2 &w, int base, const float
     // Newton (the arithmetic of newton_solve2<float>, one iteration)
     const float ax = p1x - p0x, ay = p1y - p0y, bxx = p2x - p0x, byy = p2y - p0y;
     const float exx = p3x - p1x - p2x + p0x, eyy = p3y - p1y - p2y + p0y;
-    const float det0 = diff_prod(ax, byy, bxx, ay);
+    const float det0 = ax * byy - bxx * ay;
     const float inv0 = recip_t(det0);
-    float xs = __fmul_rn(-diff_prod(p0x, byy, p0y, bxx), inv0);
-    float xt = __fmul_rn(-diff_prod(ax, p0y, ay, p0x), inv0);
-    const float j11 = __fmaf_rn(xt, exx, ax), j21 = __fmaf_rn(xt, eyy, ay);
-    const float j12 = __fmaf_rn(xs, exx, bxx), j22 = __fmaf_rn(xs, eyy, byy);
-    const float st = __fmul_rn(xs, xt);
-    const float gx = __fmaf_rn(st, exx, __fmaf_rn(xt, bxx, __fmaf_rn(xs, ax, p0x)));
-    const float gy = __fmaf_rn(st, eyy, __fmaf_rn(xt, byy, __fmaf_rn(xs, ay, p0y)));
-    const float det = diff_prod(j11, j22, j12, j21);
+    float xs = -(p0x * byy - p0y * bxx) * inv0;
+    float xt = -(ax * p0y - ay * p0x) * inv0;
+    const float j11 = ax + xt * exx, j21 = ay + xt * eyy;
+    const float j12 = bxx + xs * exx, j22 = byy + xs * eyy;
+    const float st = xs * xt;
+    const float gx = p0x + xs * ax + xt * bxx + st * exx;
+    const float gy = p0y + xs * ay + xt * byy + st * eyy;
+    const float det = j11 * j22 - j12 * j21;
     const float inv = recip_t(det);
-    const float u0 = __fmul_rn(diff_prod(gx, j22, gy, j12), inv);
-    const float u1 = __fmul_rn(diff_prod(j11, gy, j21, gx), inv);
+    const float u0 = (gx * j22 - gy * j12) * inv;
+    const float u1 = (j11 * gy - j21 * gx) * inv;
     xs -= u0;
     xt -= u1;
     const bool conv = det0 > 0.f && det > 0.f && fmaxf(fabsf(u0), fabsf(u1)) <= SL_NEWTON_TOL_F32;
-    const bool degen = det < __fmul_rn(SL_DEGENERATE, __fmul_rn(fabsf(j11) + fabsf(j21), fabsf(j12) + fabsf(j22)));
+    const bool degen = det < SL_DEGENERATE * ((fabsf(j11) + fabsf(j21)) * (fabsf(j12) + fabsf(j22)));
     const float slack = SL_SLACK_F32;
     const bool inside = xs >= -slack && xs <= 1.f + slack && xt >= -slack && xt <= 1.f + slack;
     const bool ok = in1 && conv && !degen && inside;
