@@ -29,6 +29,7 @@
 
 #include "sl_async.cuh"
 #include "sl_internal.h"
+#include "sl_newton64.cuh"
 
 namespace {
 
@@ -264,8 +265,9 @@ __device__ __forceinline__ int walk3(const Src &src, int max_iter, int walk_max,
     return ST_LOCATE;
 }
 
-// FP64 re-solve of a target whose FP32 inversion failed or whose element is nearly degenerate
-// (rare: out of line, arguments and result by value, so that the main path keeps its element and
+// FP64 solve of a target (the FP64 search of the plain kernels, sl_newton64.cuh): every target of an
+// SL_NEWTON_F64 grid, otherwise those whose FP32 inversion failed or whose element is nearly degenerate
+// (out of line, arguments and result by value, so that the main path keeps its element and
 // coordinates in registers)
 struct Resolve3 {
     int st, c0, c1, c2;
@@ -277,7 +279,6 @@ __device__ __noinline__ Resolve3 resolve3_f64(const float4 *__restrict__ D, int 
                                               int walk_max, int j0, int j1, int j2, int st32, int cx, int cy, int cz,
                                               int sx, int sy, int sz)
 {
-    const Geo3 g = {n0, n1, n2};
     const int j[3] = {j0, j1, j2};
     int c[3] = {cx, cy, cz};
     if (st32 == ST_LOCATE || st32 == ST_FOLD) {
@@ -286,10 +287,10 @@ __device__ __noinline__ Resolve3 resolve3_f64(const float4 *__restrict__ D, int 
         c[2] = sz;
     }
     double xd[3] = {0.0, 0.0, 0.0};
-    bool degd = false;
     int hops = 0, iters = 0;
-    const GlobalD3 src = {g, D};
-    const int st = walk3<double>(src, max_iter, walk_max, j, c, xd, hops, iters, &degd);
+    const int n[3] = {n0, n1, n2};
+    const int st = walk_seeded<float, 3>(reinterpret_cast<const float *>(D), n, j, max_iter, walk_max, 1e-14, 1e-12, c, xd,
+                                         &hops, &iters);
     Resolve3 r;
     r.st = st;
     r.c0 = c[0];
