@@ -921,12 +921,12 @@ def main():
         "fp64": {"value": fp64_value, "unit": UNIT, "ms_per_step": sum(ms64) / args.fp64_steps,
                  "path": "plain FP64 kernels (one thread per target, global gathers)",
                  "speedup_of_f32": value / fp64_value},
-        "roofline": {"bound": "hbm", "kernel": "remap2d_tma_kernel<32x32>, fused step (the headline's one launch per step)",
+        "roofline": {"bound": "hbm", "kernel": "gather2d_kernel<3>, fused step (the headline's one launch per step)",
                      "achieved": step_achieved, "peak": hbm, "unit": "GB/s", "frac": step_achieved / hbm,
                      "traffic": NCU_TRAFFIC["step_bytes_per_launch"] if valid else None, "peak_kind": peak_kind,
                      "algorithmic_bytes_per_launch": step_bytes, "bytes_rule": "2 F T per node (24 B)",
                      "launch_ms": step_launch_ms, "timed_over": "the headline's timed steps"},
-        "roofline_remap": {"bound": "hbm", "kernel": "remap2d_tma_kernel<32x32>, plain (sl_remap_fields)",
+        "roofline_remap": {"bound": "hbm", "kernel": "gather2d_kernel<3>, plain (sl_remap_fields)",
                            "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                            "traffic": NCU_TRAFFIC["remap_bytes_per_launch"] if valid else None, "peak_kind": peak_kind,
                            "algorithmic_bytes_per_launch": alg_bytes, "bytes_rule": "d T + 2 F T per node (32 B)",

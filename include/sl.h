@@ -177,7 +177,8 @@ typedef struct {
 
 /* Bytes of device workspace a grid needs (two displacement buffers, flags, counters and their
  * per-SM copies, reduction scratch; for the swirl and the deformation flow, sin(pi x) and
- * cos(pi x) at the node coordinates).  Returns 0 for an invalid descriptor. */
+ * cos(pi x) at the node coordinates; where the grid's default FP32 kernel reads records -- 2-D of up
+ * to 4 fields and max_order <= 1 at sizes it serves, 3-D of up to 4 fields -- 4 to 24 bytes a node).  Returns 0 for an invalid descriptor. */
 size_t sl_grid_workspace_bytes(const sl_grid_desc *desc);
 
 /* Create a grid (Sec. 2: reference mesh plus Lagrangian grid).  `dev_workspace` is caller-owned
