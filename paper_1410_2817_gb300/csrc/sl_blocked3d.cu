@@ -265,16 +265,18 @@ __device__ __forceinline__ int walk3(const Src &src, int max_iter, int walk_max,
     return ST_LOCATE;
 }
 
-// FP64 solve of a target (the FP64 search of the plain kernels, sl_newton64.cuh): every target of an
-// SL_NEWTON_F64 grid, otherwise those whose FP32 inversion failed or whose element is nearly degenerate
-// (out of line, arguments and result by value, so that the main path keeps its element and
-// coordinates in registers)
+// FP64 solve of a target, out of line, arguments and result by value, so that the main path keeps its
+// element and coordinates in registers.  SEEDED: every target of an SL_NEWTON_F64 grid, by the FP64 search
+// of the plain kernels (sl_newton64.cuh; 256^3 x 2 remap 20.1 -> 4.15 ms); otherwise the rare targets whose
+// FP32 inversion failed or whose element is nearly degenerate, by the FP64 walk (the seeded search's larger
+// frame cost the launches that hardly ever call it 1 %).
 struct Resolve3 {
     int st, c0, c1, c2;
     float x0, x1, x2;
     int hops, iters;
 };
 
+template <bool SEEDED>
 __device__ __noinline__ Resolve3 resolve3_f64(const float4 *__restrict__ D, int n0, int n1, int n2, int max_iter,
                                               int walk_max, int j0, int j1, int j2, int st32, int cx, int cy, int cz,
                                               int sx, int sy, int sz)
@@ -287,10 +289,16 @@ __device__ __noinline__ Resolve3 resolve3_f64(const float4 *__restrict__ D, int 
         c[2] = sz;
     }
     double xd[3] = {0.0, 0.0, 0.0};
-    int hops = 0, iters = 0;
-    const int n[3] = {n0, n1, n2};
-    const int st = walk_seeded<float, 3>(reinterpret_cast<const float *>(D), n, j, max_iter, walk_max, 1e-14, 1e-12, c, xd,
-                                         &hops, &iters);
+    int hops = 0, iters = 0, st;
+    if constexpr (SEEDED) {
+        const int n[3] = {n0, n1, n2};
+        st = walk_seeded<float, 3>(reinterpret_cast<const float *>(D), n, j, max_iter, walk_max, 1e-14, 1e-12, c, xd, &hops,
+                                   &iters);
+    } else {
+        bool degd = false;
+        const GlobalD3 src = {{n0, n1, n2}, D};
+        st = walk3<double>(src, max_iter, walk_max, j, c, xd, hops, iters, &degd);
+    }
     Resolve3 r;
     r.st = st;
     r.c0 = c[0];
@@ -566,7 +574,7 @@ __global__ void __launch_bounds__(NT3, 4) remap_blocked3d_kernel(const Blocked3A
         int st = ST_OK;
         if (!N64) st = walk3<float>(src, a.max_iter, a.walk_max, j, c, xf, hops, iters, &degen);
         if (N64 || st != ST_OK || degen) {
-            const Resolve3 r = resolve3_f64(a.D, g.n0, g.n1, g.n2, a.max_iter, a.walk_max, j[0], j[1], j[2], st, c[0],
+            const Resolve3 r = resolve3_f64<N64>(a.D, g.n0, g.n1, g.n2, a.max_iter, a.walk_max, j[0], j[1], j[2], st, c[0],
                                             c[1], c[2], c0[0], c0[1], c0[2]);
             st = r.st;
             c[0] = r.c0;
@@ -840,7 +848,7 @@ __global__ void __launch_bounds__(NT3, 4)
         bool degen = false;
         st = walk3<float>(src, a.max_iter, a.walk_max, j, c, xf, hops, iters, &degen);
         if (st != ST_OK || degen) {
-            const Resolve3 r = resolve3_f64(a.D, g.n0, g.n1, g.n2, a.max_iter, a.walk_max, j[0], j[1], j[2], st, c[0],
+            const Resolve3 r = resolve3_f64<false>(a.D, g.n0, g.n1, g.n2, a.max_iter, a.walk_max, j[0], j[1], j[2], st, c[0],
                                             c[1], c[2], c0[0], c0[1], c0[2]);
             st = r.st;
             c[0] = r.c0;
