@@ -116,8 +116,11 @@ typedef struct {
     const double *velocity_params;  /* host array, copied by sl_create_grid                          */
     int n_velocity_params;
     int newton_mode;                /* SL_NEWTON_F64 (any dtype) or SL_NEWTON_MIXED (SL_F32 only).
-                                       SL_F32 with SL_NEWTON_F64 inverts every target in FP64: on
-                                       the blocked kernel in 3-D, on the plain kernels in 2-D   */
+                                       SL_F32 with SL_NEWTON_F64 gives every target FP64
+                                       coordinates: on the blocked kernel in 3-D, on the plain
+                                       kernels in 2-D.  (Elements on the way are left, and Newton
+                                       started, on FP32 solutions where these are certain to
+                                       decide as FP64 does.)                                    */
     int newton_max_iter;            /* <= 0 selects 8                                                */
     int walk_max;                   /* <= 0 selects 64                                               */
     int fail_policy;                /* SL_FAIL_KEEP or SL_FAIL_ERROR                                  */
@@ -158,7 +161,8 @@ typedef struct {
     uint64_t fail_newton;           /* Newton hit its iteration cap inside the element               */
     uint64_t fail_fold;             /* det J <= 0                                                    */
     uint64_t hops_sum, hops_max;    /* element-search hops (Newton solves) per target                */
-    uint64_t iters_sum, iters_max;  /* Newton iterations per target                                  */
+    uint64_t iters_sum, iters_max;  /* Newton iterations per target, over its elements; an FP64 search
+                                       counts the FP32 ones it starts from and each FP64 pass     */
     uint64_t newton_f64;            /* (mixed mode) targets re-solved in FP64                        */
     uint64_t order_hist[3];         /* field-targets interpolated with order 0, 1, 2                 */
     uint64_t tiles_fallback;        /* tiles whose stencil window did not fit shared memory          */

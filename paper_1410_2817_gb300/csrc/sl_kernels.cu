@@ -492,8 +492,10 @@ struct BlockShape {
 // double grid, NMODE 1) run walk_seeded (sl_newton64.cuh).
 // QUINTIC: the grid may take order 2 (without it the kernel carries none of its code: the compiler
 // hoists the quintic weights out of the fields' loop, 34 FP64 instructions a target; 331 -> 264 us).
+// (Two blocks per SM for the 3-D FP64 search: left alone the compiler takes 153 registers and halves the
+// warps, 64^3 x 2 fields 176 -> 196 us.)
 template <typename T, int DIM, int NMODE, bool QUINTIC>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, DIM == 3 && NMODE <= 1 ? 2 : 0)
     remap_generic_kernel(GridArgs<T> g, const T *__restrict__ D, int ds, const uint8_t *__restrict__ flags,
                          FieldPtrs<T> f, RemapDebug<T> dbg, DevCounters *counters)
 {

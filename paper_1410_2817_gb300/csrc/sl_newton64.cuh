@@ -7,8 +7,8 @@
 // Newton iterations with their Jacobians, cofactors and divisions.  Here each element is inverted
 // in FP32 first; FP64 is used where its digits matter:
 //
-//   * an element the FP32 solution says is left by more than SEED_MARGIN needs no more digits: the
-//     walk steps on;
+//   * an element the FP32 solution says is left by more than that solution's error needs no more
+//     digits: the walk steps on;
 //   * otherwise the coordinates are polished: x <- x - Ji F(x) with the residual F in FP64 and the
 //     inverse Jacobian Ji in FP32, which gains ~6 digits per pass (two passes as a rule, 12 / 42
 //     FP64 instructions in 2-D / 3-D), down to the rounding error of F, as the FP64 iteration does.
@@ -18,10 +18,17 @@
 // 480 -> 223 us; 64^3 x 2 fields 640 -> 145 us.
 //
 // Every decision of the FP64 search (fold, no convergence, inside, next element) is taken from the
-// FP32 solution only under a certificate (seed_solve): Jacobian determinants at every iterate well
-// away from zero, iterates that stay near the element, convergence with iterations to spare.  Then
-// the FP64 iteration runs through the same points to 1e-5 and converges to the same root.  Without
-// it the element is inverted by the FP64 iteration (newton_solve), as before.
+// FP32 solution only under a certificate (seed_solve): at every iterate the columns of J exceed
+// their own rounding error by SEED_CLEAR and det J stays away from zero by more than that error can
+// move it; the steps shrink; the iteration converges with iterations to spare.  Then the FP64
+// iteration runs through nearly the same points and converges to the same root.  Without it the
+// element is inverted by the FP64 iteration (newton_solve).
+// How far the FP32 root can be from the FP64 one depends on the displacement's size (stored with 24
+// bits, a shift of 2000 cells leaves 2e-4 of a cell), on the element's shape (the inverse Jacobian
+// amplifies) and on how far outside the root lies, so a bound is formed for each coordinate (seed_clear),
+// and only coordinates beyond it decide a step.  (A fixed margin of 1e-3 lost 172 targets of a 1024^2 grid
+// displaced by 2048 cells under a shear of slope 10; the bounds cost 64^2 x 16 steps of a solid-body
+// rotation, a chain of 27 hops each, 491 -> 524 us, a 64^3 x 2 step 170 -> 176 us, 1024^2 nothing.)
 #pragma once
 
 #include <type_traits>
@@ -30,18 +37,26 @@
 
 namespace {
 
-// |det J| relative to the product of the 1-norms of J's columns (1 for a square element): above it
-// the FP32 inverse Jacobian is good to ~1e-6.
+// |det J| relative to the product of the 1-norms of J's columns (1 for a square element)
 constexpr float SEED_DET = 0.05f;
-// Iterates must stay within this distance of the element: FP32 coordinates that far out are good to
-// 128 x 6e-8 / SEED_DET ~ 2e-4, within SEED_MARGIN.  (The failing walks at the seam of a solid-body
-// rotation meet sheared elements at coordinates of 30 to 60; with 16 here a quarter of their hops
-// took the FP64 iteration, 112 against 21 us per 64^2 step.)
+// Iterates must stay within this distance of the element.  (The failing walks at the seam of a
+// solid-body rotation meet sheared elements at coordinates of 30 to 60; with 16 here a quarter of
+// their hops took the FP64 iteration, 112 against 21 us per 64^2 step.)
 constexpr float SEED_REACH = 128.f;
-// columns of J must exceed the FP32 rounding of the vertices by this factor
-constexpr float SEED_CLEAR = 1e3f;
-// distance from a face beyond which the FP32 coordinates (good to ~1e-5) decide the step
+// Columns of J must exceed the error of their entries by this factor: with entries off by e, det J
+// is off by at most DIM^2 e / column of the columns' product, 0.02 in 2-D and 0.045 in 3-D: less than
+// SEED_DET, so its sign is certain.
+constexpr float SEED_CLEAR = 200.f;
+// distance from a face beyond which the FP32 coordinates decide the step, on top of their own bound:
+// what the last Newton step (at most SL_NEWTON_TOL_F32, halved by each further one) leaves over, and
+// the room that polishing needs
 constexpr float SEED_MARGIN = 1e-3f;
+// Largest amplification of FP64 rounding (by Ji, the shape functions and the vertex coordinates) of an
+// element whose polished coordinates are a target's result.  Above it the FP64 iteration may not come
+// down to its stop, a step of 1e-14, and end as ST_NEWTON; and Map64's coefficients, rounded at the size
+// of the displacements' differences, would cost digits that the vertices of a strongly compressed element
+// have.
+constexpr float SEED_STOP = 40.f;
 // iterations the FP64 solve needs beyond the FP32 one: 3e-4 -> 1e-7 -> 1e-14 -> below its 1e-14 stop
 constexpr int SEED_SPARE = 3;
 
@@ -49,51 +64,113 @@ enum { SEED_NONE = 0, SEED_OK = 1, SEED_FOLD = 2 };
 
 template <int DIM>
 struct Seed {
-    float x[DIM];        // local coordinates
-    float Ji[DIM][DIM];  // inverse Jacobian there
+    float x[DIM];       // local coordinates
+    float C[DIM][DIM];  // cofactors of J there: the inverse is C / det
+    float det, noise;   // noise: error of a vertex coordinate and of differences of two
+    float peak[DIM];    // largest vertex coordinate along each axis
     int iters;
 };
 
-// FP32 Newton inversion of the bilinear element with vertices P (relative to the target, rounded to
-// within `noise`), the iteration of newton_solve2 under the certificate described above.
-__device__ __forceinline__ int seed_solve(const float P[4][2], float noise, int max_iter, Seed<2> &r)
+// Error of an entry of J at x, from the error `noise` of a vertex coordinate: a difference of two
+// vertices, extrapolated along the other axes (bounded by the largest coordinate).
+template <int DIM>
+__device__ __forceinline__ float entry_error(float noise, const float x[DIM])
+{
+    float far = fabsf(x[0]);
+#pragma unroll
+    for (int a = 1; a < DIM; ++a) far = fmaxf(far, fabsf(x[a]));
+    const float f = 1.f + 2.f * far;
+    return 2.f * noise * (DIM == 3 ? f * f : f);
+}
+
+// The shape functions' magnitudes at x, summed: what extrapolation does to an error of the vertices.
+template <int DIM>
+__device__ __forceinline__ float shape_sum(const float x[DIM])
+{
+    float f = 1.f;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) f *= fabsf(x[a]) + fabsf(1.f - x[a]);
+    return f;
+}
+
+// Does every coordinate lie on the same side of 0 and of 1 in FP64?  The residual at x is off by `noise`
+// times the shape sum for the vertices, and by no more than three times that for its own rounding (16
+// roundings of terms up to that sum times the largest vertex coordinate, of which `noise` holds 4); the
+// inverse Jacobian carries it into the coordinates.  (No division: this ends every hop.)
+template <int DIM>
+__device__ __forceinline__ bool seed_clear(const Seed<DIM> &s)
+{
+    const float e = 4.f * s.noise * shape_sum<DIM>(s.x);
+    bool clear = true;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        float sum = 0.f;
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) sum += fabsf(s.C[a][b]);
+        clear &= (fminf(fabsf(s.x[a]), fabsf(s.x[a] - 1.f)) - SEED_MARGIN) * s.det > sum * e;
+    }
+    return clear;
+}
+
+// Are polished coordinates inside the element as good as the FP64 iteration's?
+template <int DIM>
+__device__ __forceinline__ bool seed_final(const Seed<DIM> &s)
+{
+    float round = 0.f;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        float sum = 0.f;
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) sum += fabsf(s.C[a][b]) * fmaxf(s.peak[b], 1.f);
+        round = fmaxf(round, sum);
+    }
+    return round * shape_sum<DIM>(s.x) <= SEED_STOP * s.det;
+}
+
+// FP32 Newton inversion of the bilinear element with vertices P (relative to the target), the
+// iteration of newton_solve2 under the certificate described above (r.noise and r.peak given).
+__device__ __forceinline__ int seed_solve(const float P[4][2], int max_iter, Seed<2> &r)
 {
     const float px = P[0][0], py = P[0][1];
     const float ax = P[1][0] - px, ay = P[1][1] - py, bx = P[2][0] - px, by = P[2][1] - py;
     const float ex = P[3][0] - P[1][0] - bx, ey = P[3][1] - P[1][1] - by;
     float det = ax * by - bx * ay;
     const float na = fabsf(ax) + fabsf(ay), nb = fabsf(bx) + fabsf(by);
-    if (!(fabsf(det) > SEED_DET * (na * nb) && fminf(na, nb) > SEED_CLEAR * noise)) return SEED_NONE;
-    if (det < 0.f) return SEED_FOLD;
+    bool sure = fabsf(det) > SEED_DET * (na * nb) && fminf(na, nb) > SEED_CLEAR * 2.f * r.noise;
+    if (!(det > 0.f)) return sure ? SEED_FOLD : SEED_NONE;
     float inv = recip_t(det);
-    float s = -(px * by - py * bx) * inv, t = -(ax * py - ay * px) * inv, step = 1.f;
+    float x[2] = {-(px * by - py * bx) * inv, -(ax * py - ay * px) * inv}, step = 3e38f;
     for (int it = 0;; ++it) {
-        if (!(fabsf(s) <= SEED_REACH && fabsf(t) <= SEED_REACH)) return SEED_NONE;
-        const float j11 = ax + t * ex, j21 = ay + t * ey, j12 = bx + s * ex, j22 = by + s * ey;
+        const float j11 = ax + x[1] * ex, j21 = ay + x[1] * ey, j12 = bx + x[0] * ex, j22 = by + x[0] * ey;
         det = j11 * j22 - j12 * j21;
-        if (!(det > SEED_DET * ((fabsf(j11) + fabsf(j21)) * (fabsf(j12) + fabsf(j22))))) return SEED_NONE;
-        inv = recip_t(det);
+        const float n1 = fabsf(j11) + fabsf(j21), n2 = fabsf(j12) + fabsf(j22);
+        sure &= det > SEED_DET * (n1 * n2) && fminf(n1, n2) > SEED_CLEAR * entry_error<2>(r.noise, x) &&
+                fmaxf(fabsf(x[0]), fabsf(x[1])) <= SEED_REACH;
         if (step <= SL_NEWTON_TOL_F32) {
-            r.x[0] = s;
-            r.x[1] = t;
-            r.Ji[0][0] = j22 * inv;
-            r.Ji[0][1] = -j12 * inv;
-            r.Ji[1][0] = -j21 * inv;
-            r.Ji[1][1] = j11 * inv;
+            if (!sure) return SEED_NONE;
+            r.x[0] = x[0];
+            r.x[1] = x[1];
+            r.C[0][0] = j22;
+            r.C[0][1] = -j12;
+            r.C[1][0] = -j21;
+            r.C[1][1] = j11;
+            r.det = det;
             r.iters = it;
             return SEED_OK;
         }
-        if (it + SEED_SPARE >= max_iter) return SEED_NONE;
-        const float fx = px + s * j11 + t * bx, fy = py + s * j21 + t * by;
-        const float d0 = (fx * j22 - fy * j12) * inv, d1 = (j11 * fy - j21 * fx) * inv;
-        s -= d0;
-        t -= d1;
+        if (!sure || it + SEED_SPARE >= max_iter) return SEED_NONE;
+        inv = recip_t(det);
+        const float fx = px + x[0] * j11 + x[1] * bx, fy = py + x[0] * j21 + x[1] * by;
+        const float d0 = (fx * j22 - fy * j12) * inv, d1 = (j11 * fy - j21 * fx) * inv, last = step;
+        x[0] -= d0;
+        x[1] -= d1;
         step = fmaxf(fabsf(d0), fabsf(d1));
+        sure = step <= 0.5f * last;
     }
 }
 
 // the same for the trilinear element (vertex v = x + 2 y + 4 z)
-__device__ __forceinline__ int seed_solve(const float P[8][3], float noise, int max_iter, Seed<3> &r)
+__device__ __forceinline__ int seed_solve(const float P[8][3], int max_iter, Seed<3> &r)
 {
     float A[3][3], E01[3], E02[3], E12[3], G[3], x[3];
 #pragma unroll
@@ -107,36 +184,32 @@ __device__ __forceinline__ int seed_solve(const float P[8][3], float noise, int 
         E12[a] = P[6][a] - P[4][a] - A[a][1];
         G[a] = d76 - d54 - E01[a];
     }
-    // rows of the cofactor matrix of J give det and the inverse
-    auto invert = [](const float J[3][3], float Ji[3][3], float &det, float &norm, float &least) {
-        const float c00 = J[1][1] * J[2][2] - J[1][2] * J[2][1], c01 = J[1][2] * J[2][0] - J[1][0] * J[2][2],
-                    c02 = J[1][0] * J[2][1] - J[1][1] * J[2][0];
-        det = J[0][0] * c00 + J[0][1] * c01 + J[0][2] * c02;
+    // cofactors C of J (the inverse is C / det), det, the product of the columns' norms and the least of them
+    auto cofactors = [](const float J[3][3], float C[3][3], float &det, float &norm, float &least) {
+        C[0][0] = J[1][1] * J[2][2] - J[1][2] * J[2][1];
+        C[1][0] = J[1][2] * J[2][0] - J[1][0] * J[2][2];
+        C[2][0] = J[1][0] * J[2][1] - J[1][1] * J[2][0];
+        det = J[0][0] * C[0][0] + J[0][1] * C[1][0] + J[0][2] * C[2][0];
         const float n0 = fabsf(J[0][0]) + fabsf(J[1][0]) + fabsf(J[2][0]),
                     n1 = fabsf(J[0][1]) + fabsf(J[1][1]) + fabsf(J[2][1]),
                     n2 = fabsf(J[0][2]) + fabsf(J[1][2]) + fabsf(J[2][2]);
         norm = n0 * n1 * n2;
         least = fminf(fminf(n0, n1), n2);
-        const float inv = recip_t(det);
-        Ji[0][0] = c00 * inv;
-        Ji[1][0] = c01 * inv;
-        Ji[2][0] = c02 * inv;
-        Ji[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * inv;
-        Ji[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) * inv;
-        Ji[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) * inv;
-        Ji[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) * inv;
-        Ji[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) * inv;
-        Ji[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * inv;
+        C[0][1] = J[0][2] * J[2][1] - J[0][1] * J[2][2];
+        C[1][1] = J[0][0] * J[2][2] - J[0][2] * J[2][0];
+        C[2][1] = J[0][1] * J[2][0] - J[0][0] * J[2][1];
+        C[0][2] = J[0][1] * J[1][2] - J[0][2] * J[1][1];
+        C[1][2] = J[0][2] * J[1][0] - J[0][0] * J[1][2];
+        C[2][2] = J[0][0] * J[1][1] - J[0][1] * J[1][0];
     };
-    float det, norm, least;
-    invert(A, r.Ji, det, norm, least);
-    if (!(fabsf(det) > SEED_DET * norm && least > SEED_CLEAR * noise)) return SEED_NONE;
-    if (det < 0.f) return SEED_FOLD;
+    float C[3][3], det, norm, least;
+    cofactors(A, C, det, norm, least);
+    bool sure = fabsf(det) > SEED_DET * norm && least > SEED_CLEAR * 2.f * r.noise;
+    if (!(det > 0.f)) return sure ? SEED_FOLD : SEED_NONE;
+    float inv = recip_t(det), step = 3e38f;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) x[a] = -(r.Ji[a][0] * P[0][0] + r.Ji[a][1] * P[0][1] + r.Ji[a][2] * P[0][2]);
-    float step = 1.f;
+    for (int a = 0; a < 3; ++a) x[a] = -(C[a][0] * P[0][0] + C[a][1] * P[0][1] + C[a][2] * P[0][2]) * inv;
     for (int it = 0;; ++it) {
-        if (!(fabsf(x[0]) <= SEED_REACH && fabsf(x[1]) <= SEED_REACH && fabsf(x[2]) <= SEED_REACH)) return SEED_NONE;
         const float s01 = x[0] * x[1], s02 = x[0] * x[2], s12 = x[1] * x[2];
         float J[3][3], F[3];
 #pragma unroll
@@ -146,22 +219,32 @@ __device__ __forceinline__ int seed_solve(const float P[8][3], float noise, int 
             J[a][2] = A[a][2] + x[0] * E02[a] + x[1] * E12[a] + s01 * G[a];
             F[a] = P[0][a] + x[0] * J[a][0] + x[1] * (A[a][1] + x[2] * E12[a]) + x[2] * A[a][2];
         }
-        invert(J, r.Ji, det, norm, least);
-        if (!(det > SEED_DET * norm)) return SEED_NONE;
+        cofactors(J, C, det, norm, least);
+        sure &= det > SEED_DET * norm && least > SEED_CLEAR * entry_error<3>(r.noise, x) &&
+                fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fabsf(x[2])) <= SEED_REACH;
         if (step <= SL_NEWTON_TOL_F32) {
+            if (!sure) return SEED_NONE;
 #pragma unroll
             for (int a = 0; a < 3; ++a) r.x[a] = x[a];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) r.C[a][b] = C[a][b];
+            r.det = det;
             r.iters = it;
             return SEED_OK;
         }
-        if (it + SEED_SPARE >= max_iter) return SEED_NONE;
+        if (!sure || it + SEED_SPARE >= max_iter) return SEED_NONE;
+        inv = recip_t(det);
+        const float last = step;
         step = 0.f;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float d = r.Ji[a][0] * F[0] + r.Ji[a][1] * F[1] + r.Ji[a][2] * F[2];
+            const float d = (C[a][0] * F[0] + C[a][1] * F[1] + C[a][2] * F[2]) * inv;
             x[a] -= d;
             step = fmaxf(step, fabsf(d));
         }
+        sure = step <= 0.5f * last;
     }
 }
 
@@ -226,13 +309,27 @@ struct Map64<3> {
     }
 };
 
-// x <- x - Ji F(x) until a pass moves x by no more than 3e-11: what is left is that times the error
-// of Ji (~1e-6), below FP64 rounding.  False where it does not settle.
+// x <- x - Ji F(x), Ji the FP32 inverse Jacobian, until what a pass leaves -- its move times the bound
+// on |1 - Ji J| -- is below FP64 rounding.  The passes move x by less than SEED_MARGIN in all.  False
+// where it does not settle.
 template <int DIM>
 __device__ __forceinline__ bool polish(const Map64<DIM> &m, const Seed<DIM> &s, double x[3], int *iters)
 {
+    const float inv = recip_t(s.det);
+    float Ji[DIM][DIM], most = 0.f;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) x[a] = widen(s.x[a]);
+    for (int a = 0; a < DIM; ++a) {
+        float sum = 0.f;
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) {
+            Ji[a][b] = s.C[a][b] * inv;
+            sum += fabsf(Ji[a][b]);
+        }
+        most = fmaxf(most, sum);
+        x[a] = widen(s.x[a]);
+    }
+    // (1e-5: the rounding of Ji itself, a few 6e-8 / SEED_DET)
+    const float rate = 1e-5f + (float)DIM * most * entry_error<DIM>(s.noise, s.x);
     for (int it = 0; it < 4; ++it) {
         float F[DIM], big = 0.f;
         m.residual(x, F);
@@ -241,12 +338,12 @@ __device__ __forceinline__ bool polish(const Map64<DIM> &m, const Seed<DIM> &s, 
         for (int a = 0; a < DIM; ++a) {
             float d = 0.f;
 #pragma unroll
-            for (int b = 0; b < DIM; ++b) d += s.Ji[a][b] * F[b];
+            for (int b = 0; b < DIM; ++b) d += Ji[a][b] * F[b];
             if (!(fabsf(d) <= 0.2f * SEED_MARGIN)) return false;
             x[a] -= widen(d);
             big = fmaxf(big, fabsf(d));
         }
-        if (big <= 3e-11f) return true;
+        if (big * rate <= 1e-16f) return true;
     }
     return false;
 }
@@ -321,30 +418,34 @@ __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[
         T V[1 << DIM][DIM];
         Seed<DIM> s;
         int seed = SEED_NONE;
-        bool inner = false;  // inside the element by SEED_MARGIN (polishing moves x by less)
+        bool inner = false;  // inside the element by SEED_MARGIN and more (polishing moves x by less)
         for (;;) {
             if (hop >= walk_max) return ST_LOCATE;
             load_vertices<T, DIM>(D, n, c, V);
-            float P[1 << DIM][DIM], big = 1.f;
+            float P[1 << DIM][DIM], big = 0.f, most = 0.f;
 #pragma unroll
-            for (int v = 0; v < (1 << DIM); ++v)
+            for (int a = 0; a < DIM; ++a) {
+                s.peak[a] = 0.f;
 #pragma unroll
-                for (int a = 0; a < DIM; ++a) {
+                for (int v = 0; v < (1 << DIM); ++v) {
                     const float f = narrow(V[v][a]);
-                    big = fmaxf(big, fabsf(f));
+                    if (sizeof(T) == 8) big = fmaxf(big, fabsf(f));
                     P[v][a] = (float)(c[a] + ((v >> a) & 1) - j[a]) + f;
+                    s.peak[a] = fmaxf(s.peak[a], fabsf(P[v][a]));
                 }
-            seed = seed_solve(P, 2.4e-7f * big, max_iter, s);
+                most = fmaxf(most, s.peak[a]);
+            }
+            // 1.2e-7: the bits that narrow cuts off a double; 2.4e-7: four roundings, of P and differences
+            s.noise = 1.2e-7f * big + 2.4e-7f * most;
+            seed = seed_solve(P, max_iter, s);
             ++hop;
             *hops += 1;
             if (seed != SEED_OK) break;
             *iters += s.iters;
-            bool clear = true, out = false;
+            bool out = false;
 #pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                clear &= fabsf(s.x[a]) > SEED_MARGIN && fabsf(s.x[a] - 1.f) > SEED_MARGIN;
-                out |= s.x[a] < 0.f || s.x[a] > 1.f;
-            }
+            for (int a = 0; a < DIM; ++a) out |= s.x[a] < 0.f || s.x[a] > 1.f;
+            const bool clear = seed_clear(s);
             inner = clear && !out;
             if (!clear || !out) break;  // inside, or an axis in doubt
 #pragma unroll
@@ -361,32 +462,36 @@ __device__ __forceinline__ int walk_seeded(const T *__restrict__ D, const int n[
             for (int a = 0; a < DIM; ++a) xi[a] = NAN;
             return ST_FOLD;
         }
-        if (seed == SEED_OK) {
+        bool polished = false;
+        const bool final = seed == SEED_OK && seed_final(s);
+        if (seed == SEED_OK && (final || !inner)) {
             const int k[3] = {c[0] - j[0], c[1] - j[1], c[2] - j[2]};
             const Map64<DIM> m(V, k);
-            if (!polish<DIM>(m, s, xi, iters))
-                seed = SEED_NONE;
-            else if (inner)
-                return ST_OK;
-        }
-        if (seed == SEED_NONE) {
-            const Solved64 r = solve_element64<T, DIM>(D, n[0], n[1], n[2], c[0], c[1], c[2], j[0], j[1], j[2],
-                                                       max_iter, tol);
-            const double x[3] = {r.x0, r.x1, r.x2};
-            st = r.st;
-            *iters += r.iters;
-            bool finite = true;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                xi[a] = x[a];
-                finite &= finite_t(x[a]);
-            }
-            if (!finite) return st == ST_OK ? ST_NEWTON : st;
+            polished = polish<DIM>(m, s, xi, iters);
+            if (polished && inner) return ST_OK;
         }
         int dir[3] = {0, 0, 0};
+        for (;;) {
+            if (!polished) {
+                const Solved64 r = solve_element64<T, DIM>(D, n[0], n[1], n[2], c[0], c[1], c[2], j[0], j[1], j[2],
+                                                           max_iter, tol);
+                const double x[3] = {r.x0, r.x1, r.x2};
+                st = r.st;
+                *iters += r.iters;
+                bool finite = true;
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) dir[a] = xi[a] < -slack ? -1 : (xi[a] > 1.0 + slack ? 1 : 0);
-        if ((dir[0] | dir[1] | dir[2]) == 0) return st;
+                for (int a = 0; a < DIM; ++a) {
+                    xi[a] = x[a];
+                    finite &= finite_t(x[a]);
+                }
+                if (!finite) return st == ST_OK ? ST_NEWTON : st;
+            }
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) dir[a] = xi[a] < -slack ? -1 : (xi[a] > 1.0 + slack ? 1 : 0);
+            if ((dir[0] | dir[1] | dir[2]) != 0) break;
+            if (!polished || final) return st;
+            polished = false;
+        }
 #pragma unroll
         for (int a = 0; a < DIM; ++a) c[a] += dir[a];
         if (cyc.step(c[0], c[1], c[2])) return ST_LOCATE;
