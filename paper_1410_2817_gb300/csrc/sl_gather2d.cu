@@ -65,6 +65,7 @@ cudaError_t launch_gather2d(const sl_grid *g, const void *D, void *D_next, doubl
     A.ntiles = (int)((g->n[0] + GTX - 1) / GTX) * A.tiles_y;
     A.strips = (int)((g->n[0] + GCOLS - 1) / GCOLS);
     A.nflag = A.strips * (int)((g->n[1] + GROWS - 1) / GROWS);
+    A.hops = std::min(GHOPS, A.t.walk_max);
     A.nclaim = (A.nflag + GNT / 32 - 1) / (GNT / 32);
     VelArgs<float> vn;
     memset(&vn, 0, sizeof(vn));

@@ -29,7 +29,7 @@ namespace {
 constexpr int GMINB = 4;
 constexpr int GNT = 256;       // threads per CTA: 8 warps, one row of 32 targets each
 constexpr int GTX = 32, GTY = 8;
-constexpr int GHOPS = 4;       // elements a target of the fast path tries
+constexpr int GHOPS = 4;       // elements a target of the fast path tries (fewer under a lower hop limit)
 // nodes of a warp in phase A (2 / 4 / 8 rows: 32.6 / 30.8 / 31.8 us)
 constexpr int GCOLS = 30, GROWS = 4;
 
@@ -52,6 +52,7 @@ struct GatherArgs {
     float reach0, reach1;  // displacements of the fast path: n - 12
     int strips, nflag;   // phase A: strips of GCOLS columns, warp items
     int nclaim;          // claims of one item per warp of a CTA
+    int hops;            // the smaller of GHOPS and the grid's walk_max
 };
 
 // ---- the order of the phases --------------------------------------------------------------------
@@ -399,7 +400,7 @@ __device__ __noinline__ void general_path(const GatherArgs &A, int jx, int jy, b
     }
 }
 
-// Where one target's departure point lies: refined start, up to GHOPS elements; false where the target
+// Where one target's departure point lies: refined start, up to A.hops elements; false where the target
 // needs the general path.  (wx, wy) is the element's lower corner wrapped into the grid.
 struct Located {
     int wx, wy, hops, iters;
@@ -468,7 +469,7 @@ __device__ __forceinline__ bool locate(const GatherArgs &A, int jx, int jy, unsi
         r.xi0 = xs;
         r.xi1 = xt;
         if (xs >= -slack && xs <= 1.f + slack && xt >= -slack && xt <= 1.f + slack) return true;
-        if (r.hops == GHOPS) return false;
+        if (r.hops == A.hops) return false;
         ex += xs < -slack ? -1 : (xs > 1.f + slack ? 1 : 0);
         ey += xt < -slack ? -1 : (xt > 1.f + slack ? 1 : 0);
         wrap_cell(ex, ey, a.n0, a.n1, r.wx, r.wy);
