@@ -472,6 +472,8 @@ struct BlockShape {
         nb[1] = ((unsigned)n[1] + y - 1) / y;
         nb[2] = DIM == 2 ? 1 : ((unsigned)n[2] + z - 1) / z;
     }
+    // targets of the blocks, the places outside the grid counted in
+    unsigned long long places(unsigned threads) const { return (unsigned long long)nb[0] * nb[1] * nb[2] * threads; }
     __device__ __forceinline__ void node(unsigned block, unsigned threads, unsigned t, int j[3]) const
     {
         const unsigned r = block / nb[0], bx = block - r * nb[0];
@@ -497,7 +499,7 @@ struct BlockShape {
 template <typename T, int DIM, int NMODE, bool QUINTIC>
 __global__ void __launch_bounds__(256, DIM == 3 && NMODE <= 1 ? 2 : 0)
     remap_generic_kernel(GridArgs<T> g, const T *__restrict__ D, int ds, const uint8_t *__restrict__ flags,
-                         FieldPtrs<T> f, RemapDebug<T> dbg, DevCounters *counters)
+                         FieldPtrs<T> f, RemapDebug<T> dbg, DevCounters *counters, bool consecutive)
 {
     typedef typename std::conditional<NMODE == 1, double, T>::type TW;
     constexpr bool SEEDED = sizeof(TW) == 8;
@@ -513,8 +515,14 @@ __global__ void __launch_bounds__(256, DIM == 3 && NMODE <= 1 ? 2 : 0)
     // 1024^2 x 3 fields: 386 -> 331 us).
     __shared__ volatile double sw[sizeof(T) == 8 ? DIM * 4 : 1][sizeof(T) == 8 ? 256 : 1];
     int j[3], c[3];
-    const BlockShape<DIM> shape(g.n, blockDim.x);
-    shape.node(blockIdx.x, blockDim.x, threadIdx.x, j);
+    if (consecutive) {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        node_coords<DIM>(i, g.n, j);
+        if (i >= g.N) j[0] = g.n[0];  // past the end
+    } else {
+        const BlockShape<DIM> shape(g.n, blockDim.x);
+        shape.node(blockIdx.x, blockDim.x, threadIdx.x, j);
+    }
     const long long jj = ((long long)j[2] * g.n[1] + j[1]) * g.n[0] + j[0];
     // one pass (the loop only gives `continue` its meaning)
     for (bool todo = j[0] < g.n[0] && j[1] < g.n[1] && (DIM == 2 || j[2] < g.n[2]); todo; todo = false) {
@@ -904,36 +912,37 @@ cudaError_t Launch<T>::remap_generic(const sl_grid *g, const void *D, const uint
     // FP64 targets keep a warp busy for microseconds: a small grid is cut into small blocks, so that
     // its warps spread over the SMs
     const int NT = sizeof(T) == 4 || g->N >= 256LL * 4 * g->num_sms ? 256 : 64;
-    unsigned blocks;
-    if (g->dim == 2) {
-        const BlockShape<2> b(ga.n, NT);
-        blocks = b.nb[0] * b.nb[1];
-    } else {
-        const BlockShape<3> b(ga.n, NT);
-        blocks = b.nb[0] * b.nb[1] * b.nb[2];
-    }
+    // Blocks of targets share L1 lines (1-3 % faster on 512^2, 64^3 and 79^3); consecutive nodes where
+    // more than a tenth of the blocks' places lie outside the grid and would idle in warps that cost an
+    // FP64 instruction the same.  FP64 remaps of one field, us, consecutive / blocks: 4 x 65536 (8 places
+    // a node) 50 / 238, 33 x 8192 (1.9) 47 / 72, 48 x 8192 (1.3) 61 / 75, 28 x 16384 (1.14) 65 / 73,
+    // 512 x 512 (1) 50.6 / 49.3; 4 x 4 x 65536 (4) 318 / 1100, 14 x 64 x 400 (1.14) 127 / 137, 79^3 (1.03)
+    // 203 / 203.  FP32 on these kernels: 4 x 65536 23 / 78, 33 x 8192 25 / 31, 64^3 45 / 44.
+    const unsigned long long places = g->dim == 2 ? BlockShape<2>(ga.n, NT).places(NT) : BlockShape<3>(ga.n, NT).places(NT);
+    const bool lin = (double)places > 1.1 * (double)g->N;
+    const unsigned blocks = (unsigned)(lin ? (g->N + NT - 1) / NT : (long long)(places / NT));
     const bool n64 = g->desc.newton_mode == SL_NEWTON_F64;
     const T *d0 = (const T *)D;
     if constexpr (sizeof(T) == 8) {
         const bool z2 = g->desc.max_order > 1;
         if (g->dim == 2 && z2)
-            remap_generic_kernel<T, 2, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
         else if (g->dim == 2)
-            remap_generic_kernel<T, 2, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
         else if (z2)
-            remap_generic_kernel<T, 3, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 0, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
         else
-            remap_generic_kernel<T, 3, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 0, false><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
     } else if (g->dim == 2) {
         if (n64)
-            remap_generic_kernel<T, 2, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
         else
-            remap_generic_kernel<T, 2, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 2, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
     } else {
         if (n64)
-            remap_generic_kernel<T, 3, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 1, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
         else
-            remap_generic_kernel<T, 3, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes);
+            remap_generic_kernel<T, 3, 2, true><<<blocks, NT, 0, s>>>(ga, d0, g->ds, flags, f, d, g->stripes, lin);
     }
     return cudaGetLastError();
 }
