@@ -132,6 +132,18 @@ def percentiles(values: Sequence[float], ps=(50, 99)) -> Dict[str, float]:
 # ------------------------------------------------------------------------------------------------
 # GPU execution through the C ABI: asynchronous lanes
 # ------------------------------------------------------------------------------------------------
+def batched(wl, dtype: str) -> bool:
+    """Does the job share a batch lane?"""
+    return dtype == "f32" and wl.dim == 2 and wl.nfields <= 4 and wl.velocity not in ("carried", "nlsw")
+
+
+def grid_tile_config(wl, dtype: str, tile_config: int) -> int:
+    """Tile configuration of a job's own grid.  The batch has one of its own, and its kernels read the
+    field planes: a default grid in it would hold (and be charged) the records of the two-phase step, 8
+    to 24 bytes a node, which no call reads."""
+    return 1 if batched(wl, dtype) and tile_config == 0 else tile_config
+
+
 class Lane:
     """A unit of work the server relaunches as soon as its previous step has finished: the batch
     of all 2-D FP32 jobs with one field count, or a single other job.  Each lane owns a stream."""
@@ -170,8 +182,9 @@ class GpuExecutor:
     def bytes_of(self, job) -> int:
         sl = self.sl
         wl = job.workload
-        d = sl.make_desc(wl.dim, list(wl.n)[: wl.dim], wl.nfields, self.dtype_code(sl, job), velocity=wl.velocity,
-                         velocity_params=list(wl.velocity_params), tile_config=self.tile_config)
+        d = sl.make_desc(wl.dim, list(wl.n)[: wl.dim], wl.nfields, self.dtype_code(sl, job), max_order=wl.max_order,
+                         velocity=wl.velocity, velocity_params=list(wl.velocity_params),
+                         tile_config=grid_tile_config(wl, job.dtype, self.tile_config))
         tsize = 8 if job.dtype == "f64" else 4
         return sl.sl_grid_workspace_bytes(d) + 2 * wl.nfields * wl.nnodes * tsize
 
@@ -191,8 +204,7 @@ class GpuExecutor:
         """2-D FP32 jobs with a given velocity and at most 4 fields share a batch lane per field
         count and spline family (cubic / linear, or quintic); the others run in their own lane."""
         wl = st.job.workload
-        if (self.dtype_code(self.sl, st.job) == self.sl.SL_F32 and wl.dim == 2 and wl.nfields <= 4
-                and wl.velocity not in ("carried", "nlsw")):
+        if batched(wl, st.job.dtype):
             return ("batch", wl.nfields, wl.max_order == 2)
         return ("job", st.job.job_id)
 
@@ -211,7 +223,7 @@ class GpuExecutor:
             # FP32 work back
             prio = self.prio_fp64 if code == sl.SL_F64 else self.prio_fp32
             lane = self.lanes[key] = Lane(key, torch.cuda.Stream(priority=prio))
-        g = sl.grid_for(wl, code, tile_config=self.tile_config)
+        g = sl.grid_for(wl, code, tile_config=grid_tile_config(wl, job.dtype, self.tile_config))
         if isinstance(fields, torch.Tensor):
             f = fields.to(device="cuda", dtype=td).contiguous()
         else:

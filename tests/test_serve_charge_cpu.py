@@ -1,0 +1,30 @@
+"""What the server charges a job for (host only): the grid that it will create for it, without the records of
+kernels that a batch lane never launches."""
+import types
+
+import pytest
+
+from paper_1410_2817_gb300 import inputs
+
+
+@pytest.mark.parametrize("n", [48, 64, 200])
+def test_batched_jobs_are_not_charged_for_records(n):
+    from paper_1410_2817_gb300 import build, sl
+    from paper_1410_2817_gb300.serve import GpuExecutor
+    build.build()
+    ex = types.SimpleNamespace(sl=sl, dtype_code=GpuExecutor.dtype_code, tile_config=0)
+    for wl in (inputs.workload_swirl(n), inputs.workload_burgers(n), inputs.workload_kelvin(n)):
+        for max_order in {1, 2, wl.max_order}:
+            wl.max_order = max_order
+            planes = 2 * wl.nfields * wl.nnodes * 4
+
+            def workspace(cfg):
+                return sl.sl_grid_workspace_bytes(sl.make_desc(
+                    2, wl.n, wl.nfields, sl.SL_F32, max_order=max_order, velocity=wl.velocity,
+                    velocity_params=list(wl.velocity_params), tile_config=cfg))
+
+            charged = GpuExecutor.bytes_of(ex, inputs.Job(1, 0.0, wl, "f32")) - planes
+            # a batch lane's grid has no records; a lane of its own runs the default kernels
+            assert charged == workspace(1 if wl.velocity == "swirl2d" else 0)
+            if max_order == 2:
+                assert charged == workspace(1)
