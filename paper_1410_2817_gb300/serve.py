@@ -137,11 +137,24 @@ def batched(wl, dtype: str) -> bool:
     return dtype == "f32" and wl.dim == 2 and wl.nfields <= 4 and wl.velocity not in ("carried", "nlsw")
 
 
-def grid_tile_config(wl, dtype: str, tile_config: int) -> int:
-    """Tile configuration of a job's own grid.  The batch has one of its own, and its kernels read the
-    field planes: a default grid in it would hold (and be charged) the records of the two-phase step, 8
-    to 24 bytes a node, which no call reads."""
-    return 1 if batched(wl, dtype) and tile_config == 0 else tile_config
+def job_grid(sl, job, tile_config: int, budget: Optional[int] = None):
+    """Tile configuration of a job's own grid and the bytes the job is charged: its grid's workspace plus
+    its field and scratch planes.  The default grid holds the records of the two-phase step (2-D) or of the
+    3-D taps, 4 to 24 bytes a node.  A job goes without them (configuration 1, the same results) in a batch
+    lane, whose kernels read the field planes and take a configuration of the batch's own, and where it
+    would not fit the budget with them."""
+    wl = job.workload
+    code = sl.SL_F64 if job.dtype == "f64" else sl.SL_F32
+
+    def charge(cfg):
+        d = sl.make_desc(wl.dim, list(wl.n)[: wl.dim], wl.nfields, code, max_order=wl.max_order, velocity=wl.velocity,
+                         velocity_params=list(wl.velocity_params), tile_config=cfg)
+        return cfg, sl.sl_grid_workspace_bytes(d) + 2 * wl.nfields * wl.nnodes * (8 if code == sl.SL_F64 else 4)
+
+    if tile_config != 0 or batched(wl, job.dtype):
+        return charge(tile_config or 1)
+    full = charge(0)
+    return charge(1) if budget is not None and full[1] > budget else full
 
 
 class Lane:
@@ -171,6 +184,7 @@ class GpuExecutor:
         self.torch, self.sl = torch, sl
         self.tile_config = tile_config
         self.max_chunk = max(1, int(max_chunk))
+        self.budget = None  # bytes of the server this executor works for
         self.lanes: Dict[object, Lane] = {}
         lo, hi = torch.cuda.Stream.priority_range() if hasattr(torch.cuda.Stream, "priority_range") else (0, -1)
         self.prio_fp64, self.prio_fp32 = lo, hi  # lowest and highest priority the device offers
@@ -180,13 +194,7 @@ class GpuExecutor:
         return sl.SL_F64 if job.dtype == "f64" else sl.SL_F32
 
     def bytes_of(self, job) -> int:
-        sl = self.sl
-        wl = job.workload
-        d = sl.make_desc(wl.dim, list(wl.n)[: wl.dim], wl.nfields, self.dtype_code(sl, job), max_order=wl.max_order,
-                         velocity=wl.velocity, velocity_params=list(wl.velocity_params),
-                         tile_config=grid_tile_config(wl, job.dtype, self.tile_config))
-        tsize = 8 if job.dtype == "f64" else 4
-        return sl.sl_grid_workspace_bytes(d) + 2 * wl.nfields * wl.nnodes * tsize
+        return job_grid(self.sl, job, self.tile_config, getattr(self, "budget", None))[1]
 
     def work_of(self, job) -> float:
         """Relative device time of a job: node-steps, weighted by the measured cost of an FP64
@@ -223,7 +231,7 @@ class GpuExecutor:
             # FP32 work back
             prio = self.prio_fp64 if code == sl.SL_F64 else self.prio_fp32
             lane = self.lanes[key] = Lane(key, torch.cuda.Stream(priority=prio))
-        g = sl.grid_for(wl, code, tile_config=grid_tile_config(wl, job.dtype, self.tile_config))
+        g = sl.grid_for(wl, code, tile_config=job_grid(sl, job, self.tile_config, self.budget)[0])
         if isinstance(fields, torch.Tensor):
             f = fields.to(device="cuda", dtype=td).contiguous()
         else:
@@ -310,6 +318,7 @@ def serve_trace(jobs: Sequence, fields_of: Callable[[object], np.ndarray], budge
     """Serve a trace of inputs.Job in real time (arrival times in seconds from the start).  Returns
     latency percentiles (finish - arrival), throughput, and optionally each job's final fields."""
     ex = executor or GpuExecutor()
+    ex.budget = int(budget_bytes)
     sched = Scheduler(budget_bytes, max_active, ex.bytes_of, policy=policy, work_of=ex.work_of)
     pending = collections.deque(sorted(jobs, key=lambda j: j.arrival_s))
     results = {}
