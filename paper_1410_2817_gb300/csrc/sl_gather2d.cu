@@ -1,4 +1,6 @@
 // sl_gather2d.cu -- launches of the two-phase 2-D FP32 step (sl_gather2d.cuh).
+#include <atomic>
+
 #include "sl_gather2d.cuh"
 
 // records of a grid with n0 x n1 nodes: one plane per group, each on a 256-byte boundary
@@ -17,14 +19,14 @@ size_t gather2d_record_bytes(long long n0, long long n1, int nfields)
 template <int NF, bool FUSED>
 static cudaError_t launch_gather_nf(const sl_grid *g, GatherArgs &A, const VelArgs<float> &vn, cudaStream_t s)
 {
-    static int per_sm[64] = {};
-    int &n = per_sm[g->device & 63];
+    // CTAs per SM, looked up once per device (threads of several grids may meet here)
+    static std::atomic<int> per_sm[64];
+    int n = per_sm[g->device & 63].load(std::memory_order_relaxed);
     if (n == 0) {
-        int k = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, gather2d_kernel<NF, FUSED>, GNT, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gather2d_kernel<NF, FUSED>, GNT, 0);
         if (e != cudaSuccess) return e;
-        if (k < 1) return cudaErrorInvalidConfiguration;
-        n = k;
+        if (n < 1) return cudaErrorInvalidConfiguration;
+        per_sm[g->device & 63].store(n, std::memory_order_relaxed);
     }
     const long long ctas = std::min<long long>(A.ntiles, (long long)g->num_sms * n);
     A.step_y = (int)(ctas % A.tiles_y);
