@@ -26,7 +26,8 @@
  *     launch returns SL_ERR_CUDA (text via sl_last_error()).  Kernels never trap: a target whose
  *     element search or Newton inversion fails keeps its old value and is counted in the grid's
  *     diagnostics (read with sl_get_diagnostics); with SL_FAIL_ERROR, sl_step additionally
- *     synchronises at its end and returns SL_ERR_LOCATE / SL_ERR_NEWTON / SL_ERR_FOLD.
+ *     synchronises at its end and returns SL_ERR_LOCATE / SL_ERR_NEWTON / SL_ERR_FOLD (or SL_ERR_CUDA
+ *     if a bounded wait inside a kernel ran out: sl_diag.timeouts).
  *   - Threading: one grid is used by one stream at a time.
  *   - The library allocates no device memory: every device buffer is either the caller's field
  *     planes or the caller-supplied workspace given to sl_create_grid.
@@ -167,8 +168,11 @@ typedef struct {
     uint64_t order_hist[3];         /* field-targets interpolated with order 0, 1, 2                 */
     uint64_t tiles_fallback;        /* tiles whose stencil window did not fit shared memory          */
     uint64_t kernel_launches;       /* kernels this grid's calls have launched (host-side count)    */
-    uint64_t timeouts;              /* bounded waits for shared-memory copies that ran out (the CTA
-                                       stopped; its targets are left unwritten) -- expected 0      */
+    uint64_t timeouts;              /* thread blocks whose bounded wait ran out -- expected 0.  For
+                                       their own shared-memory copies (TMA kernels): the block
+                                       stopped and its targets are left unwritten.  For the first
+                                       phase of a two-phase 2-D step: its targets keep their old
+                                       values.  Under SL_FAIL_ERROR the call returns SL_ERR_CUDA. */
 } sl_diag;
 
 /* Remap debug outputs (device pointers, each may be NULL). */

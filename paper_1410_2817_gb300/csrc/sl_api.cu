@@ -551,6 +551,10 @@ static sl_status fail_policy_result(sl_grid *g, const DevCounters &before, cudaS
     if (after.fail_locate > before.fail_locate) return SL_ERR_LOCATE;
     if (after.fail_newton > before.fail_newton) return SL_ERR_NEWTON;
     if (after.fail_fold > before.fail_fold) return SL_ERR_FOLD;
+    if (after.timeouts > before.timeouts) {
+        snprintf(g_last_error, sizeof(g_last_error), "a bounded wait inside a kernel ran out");
+        return SL_ERR_CUDA;
+    }
     return SL_OK;
 }
 

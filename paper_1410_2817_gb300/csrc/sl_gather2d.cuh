@@ -67,25 +67,20 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// thread 0 waits (bounded: 4 s of globaltimer); the CTA learns the result
+// Thread 0 waits, for GWAITS looks at the counter (a quarter of a microsecond and more each: over 2 s;
+// looks are counted instead of time because a clock runs on while another process has the GPU); the CTA
+// learns the result.
+constexpr int GWAITS = 1 << 23;
 __device__ __forceinline__ bool wait_items(const unsigned *sync, unsigned n, int *s_ok)
 {
     if (threadIdx.x == 0) {
-        int ok = 1;
-        if (ld_acquire(sync + 1) < n) {
-            unsigned long long t0, t1;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-            while (ld_acquire(sync + 1) < n) {
-                __nanosleep(40);
-                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-                if (t1 - t0 > 4000000000ull) {
-                    ok = 0;
-                    break;
-                }
-            }
+        int left = GWAITS;
+        while (ld_acquire(sync + 1) < n && left > 0) {
+            __nanosleep(40);
+            --left;
         }
         __threadfence();
-        *s_ok = ok;
+        *s_ok = left > 0;
     }
     __syncthreads();
     return *s_ok != 0;
@@ -538,6 +533,22 @@ __device__ __forceinline__ void integrate_tiles(const GatherArgs &A, const VelAr
     }
 }
 
+// A CTA whose wait ran out: its targets from w on keep their old values.
+template <int NF, bool FUSED>
+__device__ __noinline__ void keep_old(const GatherArgs &A, TileWalk w)
+{
+    const TileArgs &a = A.t;
+    if (threadIdx.x == 0) atomicAdd(A.timeouts, 1ull);
+    for (; !w.end(A); w.next(A)) {
+        if (!w.valid(A)) continue;
+        const unsigned jj = (unsigned)w.y() * (unsigned)a.n0 + (unsigned)w.jx;
+        for (int f = 0; f < NF; ++f) a.out[f][jj] = a.in[f][jj];
+        if (FUSED && a.D_next != nullptr && a.carried)
+            reinterpret_cast<float2 *>(a.D_next)[jj] =
+                make_float2(a.csc[0] * a.in[a.vf[0]][jj], a.csc[1] * a.in[a.vf[1]][jj]);
+    }
+}
+
 template <int NF, bool FUSED>
 __global__ void __launch_bounds__(GNT, GMINB) gather2d_kernel(const __grid_constant__ GatherArgs A, const VelArgs<float> vn)
 {
@@ -577,7 +588,7 @@ __global__ void __launch_bounds__(GNT, GMINB) gather2d_kernel(const __grid_const
         if (!waited) {
             waited = true;
             if (!wait_items(A.sync, (unsigned)A.nclaim, &s_ok)) {
-                if (threadIdx.x == 0) atomicAdd(A.timeouts, 1ull);
+                keep_old<NF, FUSED>(A, w);
                 break;
             }
         }
