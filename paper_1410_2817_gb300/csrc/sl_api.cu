@@ -128,8 +128,13 @@ struct Layout {
 //                   11.6, 513^2 13.1 / 13.7);
 //   4 fields        (two records a tap) 256^2 9.5 / 11.3, 400^2 13.7 / 11.5, 1024^2 36.3 / 33.6,
 //                   1449^2 (2116) 68.0 / 63.2, 2048^2 (4096) 129 / 139: small and large grids only.
+// Oblong grids follow the same lines down to sides of 16 (16 x 16384 x 3 fields, 512 tiles: 17.5 / 20.8;
+// 100 x 1000 x 3, 128 tiles: 10.2 / 10.4).  A side below 16 leaves most lanes of the 32-wide rows idle and
+// sends displacements beyond n - 12 to the general path: 12 x 2000 x 3 14.2 / 8.0, 4 x 65536 81 / 49, 500 x 4
+// 10.1 / 4.3: never.
 bool two_phase_size(const sl_grid_desc *d, bool moving)
 {
+    if (std::min(d->n[0], d->n[1]) < 16) return false;
     const long long tiles = ((d->n[0] + 31) / 32) * ((d->n[1] + 31) / 32), wave = 456;
     if (d->nfields <= 3) return moving || tiles <= wave / 4 || tiles > wave;
     return tiles <= wave / 5 || tiles > 7 * wave;
