@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(Cfg::NT, ADVB)
             stage_factors(sg, tgrid[gid], sv.ct);
         }
         __syncthreads();
-        const bool pairs = fourier2d_pairs(sv);
+        const bool pairs = sv.pairs != 0;
         if (pairs) {
             sf.load(sv, threadIdx.x);
             __syncthreads();

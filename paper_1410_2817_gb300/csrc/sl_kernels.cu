@@ -48,6 +48,7 @@ VelArgs<T> make_vel_args(const sl_grid *g, double t, double dt)
     v.integrator = g->desc.integrator;
     v.substeps = g->desc.trajectory_substeps > 0 ? g->desc.trajectory_substeps : 1;
     for (int q = 0; q < SL_MAX_VEL_PARAMS; ++q) v.p[q] = (T)g->vel_params[q];
+    v.pairs = sizeof(T) == 4 && v.kind == SL_VEL_FOURIER2D && fourier2d_pairs(v.integrator, v.substeps, dt, g->vel_params);
     if (v.kind == SL_VEL_SWIRL2D || v.kind == SL_VEL_DEFORM3D) {
         stage_time_factors<T>(t, dt, v.substeps, v.integrator, g->vel_params[0], v.ct);
     }
@@ -248,12 +249,13 @@ __global__ void __launch_bounds__(256) advect_kernel(GridArgs<T> g, VelArgs<T> v
 }
 
 // The RK4 step of a 2-D Fourier velocity in FP32, two nodes a thread (rk4_fourier2d_pair): nodes i and
-// i + half of the grid.
-__global__ void __launch_bounds__(256, 3)
+// i + half of the grid.  NT threads a block, G modes at a time.
+template <int NT, int G>
+__global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1)
     advect_fourier2d_kernel(GridArgs<float> g, VelArgs<float> v, float2 *__restrict__ D, unsigned half)
 {
     __shared__ FourierPairs sf;
-    __shared__ float4 base[SL_PAIR_MODES][256];
+    __shared__ float4 base[SL_PAIR_MODES][NT];
     sf.load(v, threadIdx.x);
     __syncthreads();
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -265,7 +267,7 @@ __global__ void __launch_bounds__(256, 3)
     const float2 X = make_float2(node_position(v.lo[0], a[0], v.dx[0]), node_position(v.lo[0], b[0], v.dx[0]));
     const float2 Y = make_float2(node_position(v.lo[1], a[1], v.dx[1]), node_position(v.lo[1], b[1], v.dx[1]));
     float2 Dx, Dy;
-    rk4_fourier2d_pair(sf, &base[0][threadIdx.x], 256, X, Y, Dx, Dy);
+    rk4_fourier2d_pair<G>(sf, &base[0][threadIdx.x], NT, X, Y, Dx, Dy);
     D[i] = make_float2(Dx.x, Dy.x);
     if (j != i) D[j] = make_float2(Dx.y, Dy.y);
 }
@@ -849,9 +851,14 @@ cudaError_t Launch<T>::advect(const sl_grid *g, void *D, double t, double dt, cu
         }
     }
     if constexpr (sizeof(T) == 4) {
-        if (fourier2d_pairs(va)) {
+        if (va.pairs) {
+            // small launches last as long as one thread's chain: blocks of 64 spread it over more SMs, four
+            // modes at a time shorten it (8 modes, 32^2 5.1 -> 3.7 us, 400^2 9.4 -> 8.0; 512^2 10.9 either way)
             const unsigned half = (unsigned)((g->N + 1) / 2);
-            advect_fourier2d_kernel<<<(half + 255) / 256, 256, 0, s>>>(ga, va, (float2 *)D, half);
+            if (g->N >= (1LL << 18))
+                advect_fourier2d_kernel<256, 2><<<(half + 255) / 256, 256, 0, s>>>(ga, va, (float2 *)D, half);
+            else
+                advect_fourier2d_kernel<64, 4><<<(half + 63) / 64, 64, 0, s>>>(ga, va, (float2 *)D, half);
             return cudaGetLastError();
         }
     }
