@@ -136,7 +136,9 @@ bool two_phase_size(const sl_grid_desc *d, bool moving)
 {
     if (std::min(d->n[0], d->n[1]) < 16) return false;
     const long long tiles = ((d->n[0] + 31) / 32) * ((d->n[1] + 31) / 32), wave = 456;
-    if (d->nfields <= 3) return moving || tiles <= wave / 4 || tiles > wave;
+    // (a solid-body rotation tears at the seam, and the targets that fail there set the launch's length:
+    // 384^2 x 3 fields 452 / 601, 513 x 511 435 / 584)
+    if (d->nfields <= 3) return moving || tiles <= wave / 4 || tiles > wave || d->velocity_kind == SL_VEL_SOLID_BODY;
     return tiles <= wave / 5 || tiles > 7 * wave;
 }
 

@@ -309,8 +309,8 @@ __device__ __forceinline__ void refine(int jx, int jy, float2 s, float fsx, floa
 
 // One FP32 inversion of element (ex, ey) with vertex displacements d (the arithmetic of the tile
 // kernels' walk_window)
-__device__ __forceinline__ bool invert_element(const TileArgs &a, int jx, int jy, int ex, int ey, const float2 d[4],
-                                               float xf[3], int &iters)
+__device__ __forceinline__ int invert_element(const TileArgs &a, int jx, int jy, int ex, int ey, const float2 d[4],
+                                              float xf[3], int &iters, bool &degen)
 {
     const float rx0 = (float)(ex - jx), rx1 = rx0 + 1.f, ry0 = (float)(ey - jy), ry1 = ry0 + 1.f;  // exact
     float P[8][3];
@@ -323,13 +323,37 @@ __device__ __forceinline__ bool invert_element(const TileArgs &a, int jx, int jy
     P[3][0] = rx1 + d[3].x;
     P[3][1] = ry1 + d[3].y;
     int it = 0;
-    bool degen = false;
     const int st = newton_solve2<float>(P, a.max_iter, SL_NEWTON_TOL_F32, xf, &it, &degen);
     iters += it;
-    return st == ST_OK && !degen;
+    return st;
 }
 
-// The general path of one target, out of line: walks of several hops, displacements of a period, and (slow_target) the FP64 re-solve of a failed or nearly degenerate inversion.
+// The FP64 re-solve of a failed or nearly degenerate FP32 inversion, with its sums (that of slow_target)
+template <int NF>
+__device__ __noinline__ TargetOut resolve_target(const TileArgs &a, bool limit, unsigned jj, int jx, int jy, int ex, int ey)
+{
+    TargetOut r = {ST_OK, 0, 0, 1, 0};
+    const Win none = {0, 0, 0, 0};
+    double xd[3] = {0.0, 0.0, 0.0};
+    bool degen = false;
+    r.st = walk2<double>(a, none, nullptr, jx, jy, ex, ey, xd, r.hops, r.iters, degen);
+    if (r.st != ST_OK) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) a.out[f][jj] = __ldg(a.in[f] + jj);
+        return r;
+    }
+    unsigned lin_mask = a.max_order == 0 ? 0xffu : 0u;
+    if (limit) lin_mask = box_flags_global(a, ex, ey);
+    r.nlin = __popc(lin_mask & ((1u << NF) - 1u));
+    interp_global(a, jj, ex, ey, (float)xd[0], (float)xd[1], lin_mask);
+    return r;
+}
+
+// The general path of one target, out of line: walks of several hops, displacements of a period, and the
+// FP64 re-solve.  The walk is walk2<float>'s, hop by hop, with the records' sums at its end, so that a
+// target that fails goes on to its FP64 walk at once.  (Fields torn by a solid-body rotation, whose failing
+// walks of 55 hops set the launch's length, 200^2 x 3 / 1024^2 x 3: 539 / 460 us; repeating the FP32 walk in
+// slow_target 1125 / 966; tiles 704 / 621.)
 template <int NF>
 __device__ __forceinline__ TargetOut general_target(const GatherArgs &A, int jx, int jy, bool limit)
 {
@@ -346,30 +370,41 @@ __device__ __forceinline__ TargetOut general_target(const GatherArgs &A, int jx,
         load_quad(a, wrap_idx(cx, a.n0), wrap_idx(cy, a.n1), d);
         refine(jx, jy, s, fsx, fsy, d, ex, ey);
     }
-    const int rex = ex, rey = ey;
     const float slack = SL_SLACK_F32;
     TargetOut r = {ST_OK, 0, 0, 0, 0};
     CycleCheck cyc;
     cyc.start(ex, ey, 0);
+    int st = ST_LOCATE, wx = 0, wy = 0;
+    bool degen = false;
+    float xf[3];
 #pragma unroll 1
     for (int hop = 0; hop < a.walk_max; ++hop) {
-        const int wx = wrap_idx(ex, a.n0), wy = wrap_idx(ey, a.n1);
+        wx = wrap_idx(ex, a.n0);
+        wy = wrap_idx(ey, a.n1);
         load_quad(a, wx, wy, d);
-        float xf[3];
         r.hops += 1;
-        if (!invert_element(a, jx, jy, ex, ey, d, xf, r.iters)) break;
+        st = invert_element(a, jx, jy, ex, ey, d, xf, r.iters, degen);
+        if (!(finite_t(xf[0]) && finite_t(xf[1]))) {
+            if (st == ST_OK) st = ST_NEWTON;
+            break;
+        }
         const bool lo0 = xf[0] < -slack, hi0 = xf[0] > 1.f + slack;
         const bool lo1 = xf[1] < -slack, hi1 = xf[1] > 1.f + slack;
-        if (!(lo0 || hi0 || lo1 || hi1)) {
-            r.nlin = (int)target_sums<NF>(A, jj, wx, wy, xf[0], xf[1], limit);
-            return r;
-        }
+        if (!(lo0 || hi0 || lo1 || hi1)) break;
+        st = ST_LOCATE;
         ex += lo0 ? -1 : (hi0 ? 1 : 0);
         ey += lo1 ? -1 : (hi1 ? 1 : 0);
         if (cyc.step(ex, ey, 0)) break;
     }
-    const Win none = {0, 0, 0, 0};
-    return slow_target<NF>(a, none, nullptr, nullptr, 0, nullptr, limit, jj, jx, jy, rex, rey, cx, cy);
+    if (st == ST_OK && !degen) {
+        r.nlin = (int)target_sums<NF>(A, jj, wx, wy, xf[0], xf[1], limit);
+        return r;
+    }
+    const bool lost = st == ST_LOCATE || st == ST_FOLD;
+    TargetOut q = resolve_target<NF>(a, limit, jj, jx, jy, lost ? cx : ex, lost ? cy : ey);
+    q.hops += r.hops;
+    q.iters += r.iters;
+    return q;
 }
 
 // ... and its counters, added one target at a time to the SM's copy, so that the loop over the targets
