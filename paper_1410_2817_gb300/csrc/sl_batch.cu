@@ -137,10 +137,12 @@ __global__ void __launch_bounds__(CfgZ::NT, CfgZ::MINB)
     }
 }
 
-// The trajectory and the finishing kernel claim runs of up to RUN_TILES consecutive tiles of one grid: claimed
-// tile by tile they are bound by the counter (~6 ns a claim, 25,000 tiles in 512 grids of 24.4 M nodes).
-// Longer runs leave CTAs idle at the end.  The finishing copy: 138 -> 100 us.
-constexpr int RUN_TILES = 2;
+// The trajectory and the finishing kernel claim runs of consecutive tiles of one grid: claimed tile by tile
+// they are bound by the counter (~6 ns a claim, 25,000 tiles in 512 grids of 24.4 M nodes).  Longer runs leave
+// CTAs idle at the end.  The finishing copy: 138 -> 100 us.  A batch with fewer tiles than CTAs claims them
+// singly (16 grids of sides 40 to 100, a one-step call: 117 -> 97 us).
+constexpr int RUN_TILES = 2, RUN_CTAS = 8 * 152;
+constexpr int run_tiles(long long nitems) { return nitems > RUN_CTAS ? RUN_TILES : 1; }
 // CTAs per SM of the trajectory kernel's register budget (2 / 3 / 4: 773 / 702 / 724 us)
 constexpr int ADVB = 3;
 
@@ -289,7 +291,7 @@ struct sl_batch {
     unsigned *counters;
     double *tgrid;
     int nruns;
-    Run *runs;           // the tiles in runs of up to RUN_TILES of one grid
+    Run *runs;           // the tiles in runs of one grid
     std::vector<double> t_host, dt_host;
     std::vector<int> dcur0;           // displacement buffer each grid's advect writes at a call start
     unsigned long long launches = 0;  // kernels launched by this batch's calls
@@ -315,17 +317,17 @@ static int batch_cfg(sl_grid *const *grids, int tile_config)
 extern "C" size_t sl_batch_workspace_bytes(sl_grid *const *grids, int count, int tile_config)
 {
     if (!grids || count < 1 || tile_config < 0 || tile_config > 5) return 0;
-    long long nitems = 0, nruns = 0;
+    long long nitems = 0, pairs = 0;
     for (int q = 0; q < count; ++q) {
         if (!batch_eligible(grids[q])) return 0;
         if ((grids[q]->desc.max_order == 2) != (grids[0]->desc.max_order == 2)) return 0;
         int tx, ty;
         tile_counts(batch_cfg(grids, tile_config), grids[q], &tx, &ty);
         nitems += (long long)tx * ty;
-        nruns += ((long long)tx * ty + RUN_TILES - 1) / RUN_TILES;
+        pairs += ((long long)tx * ty + RUN_TILES - 1) / RUN_TILES;
     }
     if (nitems > (1LL << 30)) return 0;
-    return batch_layout(count, (int)nitems, (int)nruns).total;
+    return batch_layout(count, (int)nitems, (int)(run_tiles(nitems) == 1 ? nitems : pairs)).total;
 }
 
 extern "C" sl_status sl_batch_create(sl_grid *const *grids, int count, void *const *const *fields,
@@ -385,9 +387,9 @@ extern "C" sl_status sl_batch_create(sl_grid *const *grids, int count, void *con
     }
     b->nitems = (int)items.size();
     std::vector<Run> runs;
+    const int len = run_tiles(b->nitems);
     for (int q = 0; q < count; ++q)
-        for (int t = 0; t < table[q].ntiles; t += RUN_TILES)
-            runs.push_back({q, t, std::min(RUN_TILES, table[q].ntiles - t)});
+        for (int t = 0; t < table[q].ntiles; t += len) runs.push_back({q, t, std::min(len, table[q].ntiles - t)});
     b->nruns = (int)runs.size();
     b->L = batch_layout(count, b->nitems, b->nruns);
     b->ws = (char *)dev_workspace;
