@@ -129,8 +129,8 @@ typedef struct {
     int kernel;                     /* SL_KERNEL_AUTO, SL_KERNEL_GENERIC or SL_KERNEL_TILED           */
     int tile_config;                /* 2-D FP32 kernel: 0 default (up to 4 fields and max_order <= 1:
                                        the two-phase kernel, which flags every node once and
-                                       gathers through L1, or 1, whichever is the faster one for
-                                       the size; else 1);
+                                       gathers through L1 from records in the workspace, or 1,
+                                       whichever is the faster one for the size and flow; else 1);
                                        6: 64x32 and 7: 32x32 tiles of the persistent kernel whose
                                        windows are copied by TMA boxes (one CTA per SM with 6, two
                                        with 7; up to 3 fields, max_order <= 1, an analytic velocity,
@@ -186,7 +186,10 @@ typedef struct {
 /* Bytes of device workspace a grid needs (two displacement buffers, flags, counters and their
  * per-SM copies, reduction scratch; for the swirl and the deformation flow, sin(pi x) and
  * cos(pi x) at the node coordinates; where the grid's default FP32 kernel reads records -- 2-D of up
- * to 4 fields and max_order <= 1 at sizes it serves, 3-D of up to 4 fields -- 4 to 24 bytes a node).  Returns 0 for an invalid descriptor. */
+ * to 4 fields and max_order <= 1 at sizes it serves, 3-D of up to 4 fields -- 4 to 24 bytes a node).
+ * tile_config 1 goes without records, with the same results: for a grid that lives in a batch, whose
+ * kernels read the field planes, a 3-D one of up to 2 fields that is only ever remapped, or where memory
+ * is short.  Returns 0 for an invalid descriptor. */
 size_t sl_grid_workspace_bytes(const sl_grid_desc *desc);
 
 /* Create a grid (Sec. 2: reference mesh plus Lagrangian grid).  `dev_workspace` is caller-owned

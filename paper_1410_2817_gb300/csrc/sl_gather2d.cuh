@@ -44,7 +44,7 @@ constexpr int REC_LO = 1, REC_HI = 2;
 
 struct GatherArgs {
     TileArgs t;
-    void *rec[3];        // node (0, 0) of each group's plane
+    void *rec[2];        // node (0, 0) of each group's plane (up to four fields: two groups)
     unsigned *sync;      // claims taken, claims done, CTAs that left
     unsigned long long *timeouts;
     int tiles_y, ntiles; // GTX x GTY tiles, numbered down the columns
@@ -288,7 +288,6 @@ __device__ __forceinline__ unsigned target_sums(const GatherArgs &A, unsigned jj
     const int o = (ey - 1) * (A.t.n0 + REC_LO + REC_HI) + (ex - 1);
     target_group<NF, 0>(A, jj, o, wc, xi0, xi1, limit, nlin);
     if constexpr (rec_groups(NF) > 1) target_group<NF, 1>(A, jj, o, wc, xi0, xi1, limit, nlin);
-    if constexpr (rec_groups(NF) > 2) target_group<NF, 2>(A, jj, o, wc, xi0, xi1, limit, nlin);
     return nlin;
 }
 
