@@ -94,7 +94,6 @@ struct VelArgs {
     int nmodes;
     int integrator;   // SL_RK4 or SL_WRK3
     int substeps;     // integrator steps of dt / substeps per step (1 .. SL_MAX_SUBSTEPS)
-    int pairs;        // trajectory launches take the two-node code of a 2-D Fourier velocity
     T p[SL_MAX_VEL_PARAMS];
     // cos(pi t/T) at the stage times of sub-step s in ct[3 s + 0..2] (time-dependent flows):
     // RK4 t_s, t_s + h/2, t_s + h; WRK3 t_s, t_s + h/3, t_s + 3h/4 (h = dt / substeps)
@@ -104,6 +103,9 @@ struct VelArgs {
     // sin(pi x), cos(pi x) at the grid's node coordinates x = lo + k dx of each axis (pairs, node k
     // at 2k), tabulated once per grid for the swirl and the deformation flow; null otherwise
     const T *sc[3];
+    // trajectory launches take the two-node code of a 2-D Fourier velocity (at the end: one word further up
+    // the constants lose the alignment that their paired loads need, 256^3 x 2 step 1160 -> 1212 us)
+    int pairs;
 };
 
 template <typename T>
