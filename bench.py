@@ -43,7 +43,7 @@ FLUSH_BYTES = 512 << 20
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch at 1024^2 (3 fields) of the fused step
 # kernel (the headline's only launch) and of the plain remap kernel (sl_remap_fields), from the ncu
 # captures summarised in profiles/; valid only for the kernel source they were taken on.
-NCU_TRAFFIC = {"step_bytes_per_launch": 21531136, "remap_bytes_per_launch": 21165824, "source_sha": "3092148f233e64c9"}
+NCU_TRAFFIC = {"step_bytes_per_launch": 21519872, "remap_bytes_per_launch": 21204224, "source_sha": "8a10d3a1884bb591"}
 
 
 def warm_flushed(flush, step, n=3):
